@@ -163,7 +163,6 @@ struct Smem {
   float btri32b[2 * kBTri];
   float redh[2][kWarps / 2];
   float2 whv[kWarps][32], whw[kWarps][32];   // the same per warp (warp-level estimates, m <= 32)
-  int bcast;
   int jmode, jm, jn;          // cluster split of a bond visit: 0 none, 2 cluster Jacobi; its matrix shape (leader)
   int jflag[2];               // cluster Jacobi: a rotation happened in the sweep of this parity (leader)
   double jfro;                // cluster Jacobi: |B|_F^2 (leader)
@@ -177,6 +176,14 @@ struct Smem {
   uint64_t tc_mbar;           // tensor-core Gram: completion barrier of its MMAs
   uint32_t tc_tmem;           // its TMEM accumulator (column base)
   uint32_t tc_commits;        // commits on tc_mbar so far (its phase parity)
+  int npure, pure;            // select_class: classes of the purity test, and whether it decided (leader)
+  int vbond;                  // bond of the visit the cluster serves next, -1 to leave the sweeps (leader)
+  uint8_t clean[kMaxN];       // bond b: the state around it is the one its last visit left (leader, disentangle)
+  // the leader's counters of the launch (load_counters): one thread adds to them several times per visit, which
+  // in global memory took about 10 of the 200 kcycles of a small visit
+  long long stats[S_COUNT];
+  long long prof[P_COUNT];
+  double dstats[kDStats];
 };
 
 struct Ctx {
@@ -263,6 +270,28 @@ __device__ void set_failure(const Ctx& C, int code, int where, int a, int b) {
     C.meta[M_DIAG_A] = a;
     C.meta[M_DIAG_B] = b;
   }
+}
+
+// The leader's counters live in its shared memory while a gate-list kernel runs: fetched at its start, stored
+// at its end (dstats[3], which every CTA adds to, stays in global memory).
+__device__ void load_counters(Smem& s, Ctx& C) {
+  if (C.rank != 0) return;
+  for (int i = threadIdx.x; i < S_COUNT; i += blockDim.x) s.stats[i] = C.stats[i];
+  for (int i = threadIdx.x; i < P_COUNT; i += blockDim.x) s.prof[i] = C.prof[i];
+  if (threadIdx.x < kDStats) s.dstats[threadIdx.x] = C.dstats[threadIdx.x];
+  __syncthreads();
+  C.stats = s.stats;
+  C.prof = s.prof;
+  C.dstats = s.dstats;
+}
+__device__ void store_counters(Smem& s, const Ctx& C) {
+  if (C.rank != 0) return;
+  __syncthreads();
+  const Engine& e = *C.e;
+  for (int i = threadIdx.x; i < S_COUNT; i += blockDim.x) e.stats[(long long)C.c * S_COUNT + i] = s.stats[i];
+  for (int i = threadIdx.x; i < P_COUNT; i += blockDim.x)
+    if (i < P_SMID || i >= P_SMID + kProfSmids) e.prof[(long long)C.c * P_COUNT + i] = s.prof[i];
+  if (threadIdx.x < kDStats && threadIdx.x != 3) e.dstats[(long long)C.c * kDStats + threadIdx.x] = s.dstats[threadIdx.x];
 }
 
 static_assert((kWarps & (kWarps - 1)) == 0 && kWarps <= 32, "block_sum's shuffle tree");
@@ -910,6 +939,28 @@ __device__ void note_chi(const Ctx& C, int k) {
   if (threadIdx.x == 0 && k > C.stats[S_MAXCHI]) C.stats[S_MAXCHI] = k;
 }
 
+// A centre move over a bond of dimension 1: the centre A (m entries) is its norm times a unit tensor, and the norm
+// goes into the neighbour (m2 entries).  A zero tensor becomes e_1 with norm 0, as block_qr leaves it.
+__device__ void move_unit(Smem& s, const Ctx& C, double2* A, int m, double2* A2, int m2, int centre) {
+  // up to two entries a lane, the first warp does it alone: one barrier instead of block_qr's ten or so
+  const bool one = m <= 64;
+  if (!one || threadIdx.x < 32) {
+    const int nt = one ? 32 : (int)blockDim.x;
+    double n2 = 0;
+    for (int i = threadIdx.x; i < m; i += nt) n2 += cabs2(A[i]);
+    n2 = one ? warp_sum(n2) : block_sum(n2, s);
+    const double nrm = sqrt(n2), inv = n2 > 0.0 ? 1.0 / nrm : 0.0;
+    for (int i = threadIdx.x; i < m; i += nt)
+      A[i] = n2 > 0.0 ? cscale(A[i], inv) : make_double2(i == 0 ? 1.0 : 0.0, 0.0);
+    for (int i = threadIdx.x; i < m2; i += nt) A2[i] = cscale(A2[i], nrm);
+  }
+  if (threadIdx.x == 0) {
+    C.stats[S_QR] += 1;
+    C.meta[M_OC] = centre;
+  }
+  __syncthreads();
+}
+
 // Centre j -> j+1 without truncation (Sec. 2.4 canonical form): A_j = Q R (reduced QR of the
 // (chi_l d) x chi_r matrix), A_j <- Q, A_{j+1} <- R A_{j+1}; the bond keeps min(chi_l d, chi_r).
 __device__ void move_right(Smem& s, const Ctx& C, int j) {
@@ -918,6 +969,10 @@ __device__ void move_right(Smem& s, const Ctx& C, int j) {
   const int cl = C.dims[j], cr = C.dims[j + 1], cr2 = C.dims[j + 2];
   double2* A = site_ptr(C, j);
   double2* A2 = site_ptr(C, j + 1);
+  if (cr == 1) {
+    move_unit(s, C, A, cl * d, A2, d * cr2, j + 1);
+    return;
+  }
   double2* B = C.scr + e.sl.b;
   double2* Q = C.scr + e.sl.u;
   double2* R = C.scr + e.sl.vh;
@@ -953,6 +1008,10 @@ __device__ void move_left_qr(Smem& s, const Ctx& C, int j) {
   const int cl = C.dims[j], cr = C.dims[j + 1], cl2 = C.dims[j - 1];
   double2* A = site_ptr(C, j);
   double2* A0 = site_ptr(C, j - 1);
+  if (cl == 1) {
+    move_unit(s, C, A, d * cr, A0, cl2 * d, j - 1);
+    return;
+  }
   double2* B = C.scr + e.sl.b;
   double2* Q = C.scr + e.sl.u;
   double2* R = C.scr + e.sl.vh;
@@ -1807,7 +1866,7 @@ __device__ __noinline__ Score score_class_fp32(const Grp& g, const Ctx& C, int c
 template <class Grp>
 __device__ Score score_class(const Grp& g, const Ctx& C, const double2* theta, int cl, int cr, const double2* Q,
                              const float2* Q32, double2* ws, long long gram_off, bool want_vn, double* tri,
-                             float* tri32, int tricap) {
+                             float* tri32, int tricap, bool force64 = false) {
   const int d = C.d, dd = d * d;
   const int rows = cl * d, cols = d * cr;
   const int m = rows < cols ? rows : cols;
@@ -1815,7 +1874,7 @@ __device__ Score score_class(const Grp& g, const Ctx& C, const double2* theta, i
   double2* G = ws + gram_off;
   double* dg = reinterpret_cast<double*>(G + (long long)m * m);
   double* od = dg + m;
-  if (C.e->precision && m > kPruneMin && Q != C.e->candU)
+  if (!force64 && C.e->precision && m > kPruneMin && Q != C.e->candU)
     return score_class_fp32(g, C, cl, cr, Q32, ws, gram_off, want_vn, tri, tri32, tricap);
   // the leader's own exact evaluations, timed part by part (thread 0: warp 0's or the CTA's)
   long long* xw = (want_vn && C.prof && C.rank == 0 && threadIdx.x == 0)
@@ -2424,7 +2483,8 @@ __device__ __noinline__ bool gram_tc(Smem& s, const Ctx& C, const float2* X, int
   __syncthreads();
   if (tid == 0) {
     s.tc_commits = commits;
-    if (C.dstats) C.dstats[3] += 8.0 * m * m * Kc;   // algorithmic flops of the complex Gram
+    // algorithmic flops of the complex Gram (every CTA of the cluster adds its own)
+    if (C.dstats) atomicAdd(C.e->dstats + (long long)C.c * kDStats + 3, 8.0 * m * m * Kc);
   }
   if (!ok && tid == 0) set_failure(C, GCAMPS_ENOCONV, 3, rows, cols);
   __syncthreads();
@@ -2474,8 +2534,9 @@ __device__ void gram_fp32<BlockGroup>(const BlockGroup& g, const Ctx& C, const f
 // one class per warp, large ones one class per CTA.  Results go to the leader CTA's shared memory.
 // mode kExact: S2 and S_vN in FP64; kScreen: S2 in FP32 with its lower bound (lead->s2lo).
 // kS2Exact: S2 in FP64 only (class 0 still gets kExact: its eigenvalues certify QR moves).
+// kPurity: S2 in FP64 only, for every listed class and in the precision form too.
 // kEstimate: the FP32 von Neumann estimate and its bound (lead->vest, lead->vbd; CTA-level sizes only).
-enum ScoreMode { kExact = 0, kScreen = 1, kS2Exact = 2, kEstimate = 3 };
+enum ScoreMode { kExact = 0, kScreen = 1, kS2Exact = 2, kEstimate = 3, kPurity = 4 };
 __device__ void score_classes(Smem& s, Smem* lead, const Ctx& C, const double2* theta, int cl, int cr,
                               const int* list, int cnt, int mode) {
   const Engine& e = *C.e;
@@ -2517,11 +2578,11 @@ __device__ void score_classes(Smem& s, Smem* lead, const Ctx& C, const double2* 
         }
         continue;
       }
-      const bool want_vn = mode == kExact || k == 0;
+      const bool want_vn = mode == kExact || (mode == kS2Exact && k == 0);
       const long long t0 = (C.prof && C.rank == 0 && warp == 0 && lane == 0) ? clock64() : 0;
       const Score sc = score_class(g, C, theta, cl, cr, e.candU + (long long)k * dd * dd,
                                    e.candU32 + (long long)k * dd * dd, ws, kSmall, want_vn, s.wtri[warp],
-                                   s.wtri32[warp], 32);
+                                   s.wtri32[warp], 32, mode == kPurity);
       if (C.prof && C.rank == 0 && warp == 0 && lane == 0 && want_vn) {   // the leader's own exact evaluations
         C.prof[P_LEAD_EXACT_CYC] += clock64() - t0;
         C.prof[P_LEAD_EXACT_N] += 1;
@@ -2586,9 +2647,10 @@ __device__ void score_classes(Smem& s, Smem* lead, const Ctx& C, const double2* 
         __syncthreads();
         continue;
       }
-      const bool want_vn = mode == kExact || k == 0;
+      const bool want_vn = mode == kExact || (mode == kS2Exact && k == 0);
       const Score sc = score_class(g, C, theta, cl, cr, e.candU + (long long)k * dd * dd,
-                                   e.candU32 + (long long)k * dd * dd, ws, e.scap, want_vn, s.btri, s.btri32, kBTri);
+                                   e.candU32 + (long long)k * dd * dd, ws, e.scap, want_vn, s.btri, s.btri32, kBTri,
+                                   mode == kPurity);
       if (threadIdx.x == 0) {
         lead->s2[k] = sc.s2;
         lead->evald[k] = 1;
@@ -2604,13 +2666,35 @@ __device__ void score_classes(Smem& s, Smem* lead, const Ctx& C, const double2* 
 
 
 // ---------------------------------------------------------------- disentangling sweeps (Sec. 3)
+// The visit's scores (and a small theta) for gcamps_get_last_scores and gcamps_get_last_theta; leader only.
+__device__ void record_scores(Smem& s, const Ctx& C, const double2* theta, int cl, int cr) {
+  const Engine& e = *C.e;
+  const int rows = cl * C.d, cols = C.d * cr;
+  double* out = e.lastsc + (long long)C.c * (3 * kMaxK + 2 + 2 * kSmall);
+  for (int k = threadIdx.x; k < C.K; k += blockDim.x) {
+    out[k] = s.s2[k];
+    out[kMaxK + k] = s.vn[k];
+    out[2 * kMaxK + k] = s.evald[k];
+  }
+  if (threadIdx.x == 0) {
+    out[3 * kMaxK] = cl;
+    out[3 * kMaxK + 1] = cr;
+  }
+  if ((long long)rows * cols <= kSmall)
+    for (int k = threadIdx.x; k < rows * cols; k += blockDim.x) {
+      out[3 * kMaxK + 2 + 2 * k] = theta[k].x;
+      out[3 * kMaxK + 3 + 2 * k] = theta[k].y;
+    }
+}
+
 // One bond.  The leader CTA forms theta = A_i A_{i+1}; the cluster scores the classes; the leader
-// decides, applies and splits.  With the Renyi-2 bound (S2 <= S_vN): phase A gives S2 of every class
-// from an FP32 screen with a rigorous lower bound s2lo (s2_fp32), and the passes below use s2lo;
-// the first pass evaluates S_vN of the identity and of the classes with the smallest S2 (as many as the
-// cluster evaluates at once), giving an upper bound B on the best entropy; the second pass evaluates every
-// other class with S2 <= B + tie_tol (usually none: they are a prefix of the S2 order).  A class left out
-// has S_vN >= S2 > best + tie_tol, so the decision equals the one from evaluating every class.
+// decides, applies and splits.  S2 of every class comes from an FP32 screen with a rigorous lower bound s2lo
+// (s2_fp32).  If it finds classes that make theta' a product, their FP64 S2 decides (pure_choice).  Otherwise,
+// for the von Neumann score, FP32 estimates with an error bound, then exact entropies of the classes the bounds
+// cannot separate; for the other scores the first pass evaluates the identity and the classes with the smallest
+// S2 (as many as the cluster evaluates at once), giving an upper bound B on the best score; the second pass
+// every other class with S2 <= B + tie_tol.  A class left out has S_vN >= S2 > best + tie_tol, so the decision
+// equals the one from evaluating every class.
 // Cluster-wide choice of the class for one theta (shape chi_l x d x d x chi_r in global memory,
 // readable by every CTA).  Returns the chosen class on the leader (-1 on the other CTAs); the
 // leader's s.vn / s.evald hold the evaluated entropies and *nev their count.
@@ -2619,8 +2703,7 @@ __device__ void score_classes(Smem& s, Smem* lead, const Ctx& C, const double2* 
 __device__ int decide_class(Smem& s, const Ctx& C, const double2* theta, int cl, int cr, int* nev_out, long long& tp) {
   const Engine& e = *C.e;
   const bool leader = C.rank == 0;
-  const int d = C.d, kind = e.score_kind;
-  const int rows = cl * d, cols = d * cr;
+  const int kind = e.score_kind;
   if (!leader) return -1;
   if (threadIdx.x < 32) {
     // the decision over the exactly evaluated classes, on the first warp: key = S_vN (kind 0), S2 (kind 1),
@@ -2656,30 +2739,56 @@ __device__ int decide_class(Smem& s, const Ctx& C, const double2* theta, int cl,
       s.ival[5] = nev;
     }
   }
-  {
-    double* out = e.lastsc + (long long)C.c * (3 * kMaxK + 2 + 2 * kSmall);
-    for (int k = threadIdx.x; k < C.K; k += blockDim.x) {
-      out[k] = s.s2[k];
-      out[kMaxK + k] = s.vn[k];
-      out[2 * kMaxK + k] = s.evald[k];
-    }
-    if (threadIdx.x == 0) {
-      out[3 * kMaxK] = cl;
-      out[3 * kMaxK + 1] = cr;
-    }
-    if ((long long)rows * cols <= kSmall)
-      for (int k = threadIdx.x; k < rows * cols; k += blockDim.x) {
-        out[3 * kMaxK + 2 + 2 * k] = theta[k].x;
-        out[3 * kMaxK + 3 + 2 * k] = theta[k].y;
-      }
-  }
+  record_scores(s, C, theta, cl, cr);
   __syncthreads();
   prof_lap(C, P_DECIDE, tp);
   *nev_out = s.ival[5];
   return s.ival[4];
 }
 
-__device__ int select_class(Smem& s, Smem* lead, const Ctx& C, const double2* theta, int cl, int cr, int* nev_out) {
+// The purity test of the von Neumann search, on the leader's first warp once the listed classes' S2 is known in
+// FP64 (kPurity).  A theta' of rank one to rounding has S2 <= slack, slack four times the FP64 counterpart of the
+// screen's eta (the Frobenius norm of such a Gram equals its trace) plus the sums' rounding; 1 - p_0 <= S2, so
+// its entropy is at most vb = x (1 - ln x + ln m), x the bound on S2.  When vb is well below tie_tol, every such
+// class is within tie_tol of the best score; every other class lies above it if its S2 (a lower bound of S_vN)
+// does, and the classes outside the list do (s2lo > kPureList).  The choice is then the lowest such class,
+// without any eigenvalues.  Returns false (nothing decided) if there is none or a class lies in between.
+constexpr double kPureList = 1e-3;
+__device__ __forceinline__ bool pure_choice(Smem& s, const Ctx& C, int m, int M) {
+  const int lane = threadIdx.x & 31, d = C.d, np = s.npure;
+  const float u = 1.1102230e-16f, mm = (float)m * m;
+  const float slack = (4.f * (2.f * d * (d * d + 6) + 2.f * M + 4.f) + 2.f * (mm / 64.f + 16.f) + 64.f) * u;
+  const float x = 2.f * slack + 1e-13f;
+  const double vb = (double)(x * (1.f - logf(x) + logf((float)m)) * 1.01f);
+  if (!(vb <= 0.5 * C.e->tie_tol)) return false;
+  const double lo = (double)(slack + 1e-13f), hi = C.e->tie_tol + vb + 1e-11;
+  int kb = 1 << 30;
+  bool between = false;
+  for (int t = lane; t < np; t += 32) {
+    const int k = s.list[t];
+    const double v = s.s2[k];
+    const bool is_pure = v <= lo;
+    between |= !is_pure && !(v > hi);
+    if (is_pure) kb = min(kb, k);
+    s.evald[k] = is_pure;
+    s.vn[k] = v > 0.0 ? v : 0.0;
+    s.rk[k] = 1;
+  }
+  kb = warp_min_int(kb);
+  if (__any_sync(0xffffffffu, between) || kb == (1 << 30)) return false;
+  if (lane == 0) {
+    s.ival[4] = kb;
+    s.ival[5] = np;
+    s.ival[7] = 1;
+    if (kb == 0) s.rank0 = x < 1e-12f ? 1 : -1;   // the other weights are below x
+  }
+  return true;
+}
+
+// search: a disentangler visit; false for the scoring entry points, which report how many classes the
+// bounds alone leave.
+__device__ int select_class(Smem& s, Smem* lead, const Ctx& C, const double2* theta, int cl, int cr, int* nev_out,
+                            bool search) {
   long long tp = prof_start(C);
   const Engine& e = *C.e;
   const bool leader = C.rank == 0;
@@ -2702,7 +2811,50 @@ __device__ int select_class(Smem& s, Smem* lead, const Ctx& C, const double2* th
         C.th32[i] = make_float2((float)theta[i].x, (float)theta[i].y);
     cluster_sync();
   }
-  if (est_kind && small && lead->dval[3] < 1.0) {
+  // First the classes that make theta' a product across the bond (about 80 % of the visits that apply a class on
+  // the benchmark circuits): the FP32 screen finds them, their FP64 S2 settles them (pure_choice).  A Gram
+  // instead of a Gram, its reduction and its eigenvalues: 15 instead of 68 kcycles a class at m = 9.
+  const bool screened = search && est_kind && e.tie_tol >= 1e-12 && e.tie_tol <= 1e-4;
+  if (screened) {
+    score_classes(s, lead, C, theta, cl, cr, nullptr, C.K, kScreen);
+    cluster_sync();
+    prof_lap(C, P_SCREEN, tp);
+    if (leader && threadIdx.x < 32) {
+      double lo = 1e300;
+      for (int k = threadIdx.x; k < C.K; k += 32) {
+        s.evald[k] = 0;
+        lo = fmin(lo, s.s2[k]);
+      }
+      const int np = warp_min_double(lo) <= kPureList
+                         ? warp_list(s.list, 0, C.K, 0, [&](int k) { return s.s2lo[k] <= kPureList; }) : 0;
+      if (threadIdx.x == 0) {
+        s.npure = np;
+        s.pure = 0;
+      }
+    }
+    cluster_sync();
+    const int np = lead->npure;
+    if (np > 0) {
+      score_classes(s, lead, C, theta, cl, cr, lead->list, np, kPurity);
+      cluster_sync();
+      if (leader && threadIdx.x < 32) {
+        const bool done = pure_choice(s, C, m, rows < cols ? cols : rows);
+        if (threadIdx.x == 0) s.pure = done;
+      }
+      cluster_sync();
+      prof_lap(C, P_EXACT, tp);
+      if (lead->pure) {
+        if (!leader) return -1;
+        record_scores(s, C, theta, cl, cr);
+        __syncthreads();
+        prof_lap(C, P_DECIDE, tp);
+        *nev_out = s.ival[5];
+        return s.ival[4];
+      }
+    }
+  }
+  // the warp-level shortcut below estimates every class at once: for clusters with a warp per class
+  if (est_kind && small && lead->dval[3] < 1.0 && (!screened || C.csize * kWarps >= C.K)) {
     // Warp-level sizes: one pass gives every class its FP32 von Neumann estimate (and its Renyi-2 value and
     // bound, from the same Gram); exact FP64 entropies only for the identity and the classes whose estimate
     // interval reaches down to U + tie_tol, U the smallest upper bound.  A class left out has S_vN above
@@ -2731,9 +2883,11 @@ __device__ int select_class(Smem& s, Smem* lead, const Ctx& C, const double2* th
     prof_lap(C, P_EXACT, tp);
     return decide_class(s, C, theta, cl, cr, nev_out, tp);
   }
-  score_classes(s, lead, C, theta, cl, cr, nullptr, C.K, prune ? kScreen : kExact);
-  cluster_sync();
-  prof_lap(C, prune ? P_SCREEN : P_EXACT, tp);
+  if (!screened) {
+    score_classes(s, lead, C, theta, cl, cr, nullptr, C.K, prune ? kScreen : kExact);
+    cluster_sync();
+    prof_lap(C, prune ? P_SCREEN : P_EXACT, tp);
+  }
   // weight-rank threshold (the same as the QR-move certificate) and the rank lower bound from S2:
   // the weights above tau carry at least 1 - m tau of the trace, so sum p^2 >= (1 - m tau)^2 / rank and
   // rank >= exp(S2 + 2 ln(1 - m tau)) >= exp(S2 - 2.01 m tau)
@@ -2751,10 +2905,10 @@ __device__ int select_class(Smem& s, Smem* lead, const Ctx& C, const double2* th
   // tie_tol (the class that set U is evaluated exactly), so the decision equals evaluating every class.
   // the estimate bound depends on the shape only: computed once, on the leader, and read from its shared
   // memory by every CTA after the next cluster barrier
-  const bool estimate = est_kind && !small && lead->dval[3] < 1.0;
+  const bool estimate = est_kind && (!small || screened) && lead->dval[3] < 1.0;
   if (estimate) {
     if (leader) {
-      const int L = C.csize - 1;
+      const int L = (small ? C.csize * kWarps : C.csize) - 1;   // as many as run at once
       for (int k = threadIdx.x; k < C.K; k += blockDim.x) {
         s.evald[k] = 0;
         s.estd[k] = 0;
@@ -2887,36 +3041,109 @@ __device__ int select_class(Smem& s, Smem* lead, const Ctx& C, const double2* th
   return decide_class(s, C, theta, cl, cr, nev_out, tp);
 }
 
-__device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, int* accepted) {
+// The counters of a finished visit.
+__device__ __forceinline__ void end_visit(const Ctx& C, int m, long long tv) {
+  if (prof_thread(C)) {
+    C.prof[P_VCYC + prof_bucket(m)] += clock64() - tv;
+    C.prof[P_CURB] = 0;
+  }
+}
+__device__ __forceinline__ void record_decision(const Ctx& C, int i, int kb) {
+  const int nd = C.meta[M_NDEC];
+  if (nd < kDecCap) {
+    C.dec[2 * nd] = i;
+    C.dec[2 * nd + 1] = kb;
+  }
+  C.meta[M_NDEC] = nd + 1;
+}
+// FP64 flops of one exact class score (the count gcamps.h states)
+__device__ __forceinline__ void class_flops(int d, int rows, int cols, double& gram, double& tri) {
+  const long long m = rows < cols ? rows : cols, M = rows < cols ? cols : rows;
+  gram = (double)(8LL * d * d * rows * cols + 4 * m * (m + 1) * M);
+  tri = (double)(16 * m * m * m) / 3.0;
+}
+
+// What the other CTAs of the cluster do in a sweep: score the classes of the bonds that the leader publishes, and
+// rotate its big splits, until it leaves the sweeps.  The leader's visits without scoring cost no barrier.
+__device__ void serve_visits(Smem& s, Smem* lead, const Ctx& C) {
   const Engine& e = *C.e;
-  const bool leader = C.rank == 0;
+  const bool replay = e.replay && e.replay_n[C.c] > 0;
+  for (;;) {
+    cluster_sync();
+    const int i = lead->vbond;
+    if (i < 0) return;
+    const int cl = C.dims[i], cr = C.dims[i + 2];
+    int nev = 0;
+    if (!replay) select_class(s, lead, C, C.scr + e.sl.theta, cl, cr, &nev, true);
+    if (C.d * min(cl, cr) >= kClusterJacobiMin) {
+      cluster_sync();
+      if (lead->jmode == 2) jacobi_cluster(lead, C, C.scr + e.sl.b, lead->jm, lead->jn, C.scr + e.sl.w, e.jacobi_cap);
+    }
+  }
+}
+
+// One bond visit, on the leader.  must_score: the visit's scores are readable afterwards, so they are taken even
+// where the decision is known.
+__device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, bool must_score, int* accepted) {
+  const Engine& e = *C.e;
   const int d = C.d, dd = d * d;
   double2* theta = C.scr + e.sl.theta;
   double2* tmp = C.scr + e.sl.tmp;
   const long long tv = prof_start(C);
   long long tp = tv;
-  if (prof_thread(C)) {
-    const int ml = C.dims[i] * d, mr = d * C.dims[i + 2];
-    C.prof[P_CURB] = 1 + prof_bucket(ml < mr ? ml : mr);
-  }
-  if (leader) {
-    const int cl0 = C.dims[i], ch = C.dims[i + 1], cr0 = C.dims[i + 2];
-    block_matmul(theta, site_ptr(C, i), site_ptr(C, i + 1), cl0 * d, ch, d * cr0);
-    if (threadIdx.x == 0) s.rank0 = -1;
-  }
-  cluster_sync();
-  prof_lap(C, P_THETA, tp);
-  const int cl = C.dims[i], cr = C.dims[i + 2];
+  const int cl = C.dims[i], chim = C.dims[i + 1], cr = C.dims[i + 2];
   const int rows = cl * d, cols = d * cr;
   const int m = rows < cols ? rows : cols;
-  int nev = 0;
+  const int bb = C.bond_bound[i + 1];
+  const int cap = e.chi_max < bb ? e.chi_max : bb;
+  const bool replay = e.replay && e.replay_n[C.c] > 0;
+  if (prof_thread(C)) {
+    C.prof[P_CURB] = 1 + prof_bucket(m);
+    C.prof[P_VISITS + prof_bucket(m)] += 1;
+  }
+  // Two kinds of visit apply nothing whatever the classes' scores (60 % of the visits on the benchmark circuits):
+  // a bond of dimension 1 has entropy 0, which no class lowers; and around a clean bond nothing has changed since
+  // its last visit but unitaries on one side of the pair's two sites, which leave every class's score as it was
+  // (the classes of Q theta are those of theta, so after applying the best one the identity is the best).  The
+  // QR move is what a scored visit would do: the rank of the first kind is 1, the clean mark holds the second's.
+  if (!replay && !must_score && chim <= cap && (chim == 1 || s.clean[i])) {
+    if (threadIdx.x == 0) {
+      C.stats[S_BONDS] += 1;
+      C.stats[S_CANDS] += C.K;
+      if (m > kPruneMin) {
+        double gram, tri;
+        class_flops(d, rows, cols, gram, tri);
+        C.dstats[4] += C.K * (gram + tri);
+      }
+      record_decision(C, i, 0);
+    }
+    if (ltr) move_right(s, C, i);
+    else move_left_qr(s, C, i + 1);
+    note_chi(C, chim);
+    __syncthreads();
+    prof_lap(C, P_QRMOVE, tp);
+    end_visit(C, m, tv);
+    return;
+  }
+  block_matmul(theta, site_ptr(C, i), site_ptr(C, i + 1), rows, chim, cols);
+  if (threadIdx.x == 0) {
+    s.rank0 = -1;
+    s.vbond = i;
+    s.ival[7] = 0;   // 1: the purity test decided
+  }
   // Splits with many Jacobi columns run their rotations on the whole cluster: the other CTAs wait for the
   // leader's choice (a QR move or such a split) at one more cluster barrier.
   const bool big = C.csize > 1 && m >= kClusterJacobiMin;
-  if (e.replay && e.replay_n[C.c] > 0) {
-    // replay: the recorded class of this visit (every CTA reads the same list; a visit past its end or at
-    // another bond invalidates the circuit)
-    if (leader && threadIdx.x == 0) {
+  int nev = 0;
+  if (!replay) {
+    cluster_sync();
+    prof_lap(C, P_THETA, tp);
+    select_class(s, lead, C, theta, cl, cr, &nev, true);
+  } else {
+    if (big) cluster_sync();
+    // replay: the recorded class of this visit (a visit past the list's end or at another bond invalidates the
+    // circuit)
+    if (threadIdx.x == 0) {
       const int nd = C.meta[M_NDEC];
       const int* rp = e.replay + ((long long)C.c * kDecCap + nd) * 2;
       int kb = 0;
@@ -2927,45 +3154,26 @@ __device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, i
       s.rank0 = -1;   // no certificate: the visit splits by SVD
     }
     __syncthreads();
-    nev = -1;
-  }
-  const int kbsel = nev < 0 ? (leader ? s.ival[4] : -1)
-                            : select_class(s, lead, C, theta, cl, cr, &nev);
-  if (nev < 0) nev = 0;
-  if (!leader) {
-    if (!big) return;
-    cluster_sync();
-    if (lead->jmode == 2) jacobi_cluster(lead, C, C.scr + e.sl.b, lead->jm, lead->jn, C.scr + e.sl.w, e.jacobi_cap);
-    return;
+    prof_lap(C, P_THETA, tp);
   }
   tp = prof_start(C);
-  // visit counters of the size bucket; the visit's cycles are added when it ends
   if (prof_thread(C)) {
     const int b = prof_bucket(m);
-    C.prof[P_VISITS + b] += 1;
     C.prof[P_VEXACT + b] += nev;
     C.prof[P_VEST + b] += s.ival[6];
   }
   if (threadIdx.x == 0) {
-    const int kb = kbsel;
     C.stats[S_BONDS] += 1;
     C.stats[S_CANDS] += C.K;
     C.stats[S_VN] += nev;
-    {
-      const double R = rows, Cc = cols, mm = m, M = rows < cols ? cols : rows;
-      const double per_class = 8.0 * dd * R * Cc + 4.0 * mm * (mm + 1.0) * M;
-      const double tri = (16.0 / 3.0) * mm * mm * mm;
-      // exact evaluations, FP64 (Renyi-2 scores need no eigenvalues except the identity's)
-      C.dstats[1] += e.score_kind == 1 ? nev * per_class + tri : nev * (per_class + tri);
-      if (m > kPruneMin) C.dstats[4] += C.K * (per_class + tri);   // every class scored exactly (the algorithm)
-      if (m > kPruneMin) C.dstats[2] += C.K * per_class;                // FP32 screen of every class
-    }
-    const int nd = C.meta[M_NDEC];
-    if (nd < kDecCap) {
-      C.dec[2 * nd] = i;
-      C.dec[2 * nd + 1] = kb;
-    }
-    C.meta[M_NDEC] = nd + 1;
+    double gram, tri;
+    class_flops(d, rows, cols, gram, tri);
+    // exact evaluations, FP64 (Renyi-2 scores and the purity test need no eigenvalues, but for the identity's
+    // of the former)
+    C.dstats[1] += e.score_kind == 1 ? nev * gram + tri : nev * (s.ival[7] ? gram : gram + tri);
+    if (m > kPruneMin) C.dstats[4] += C.K * (gram + tri);   // every class scored exactly (the algorithm)
+    if (m > kPruneMin) C.dstats[2] += C.K * gram;                // FP32 screen of every class
+    record_decision(C, i, s.ival[4]);
   }
   __syncthreads();
   const int kb = s.ival[4];
@@ -2983,17 +3191,18 @@ __device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, i
     block_copy(theta, tmp, total);
     __syncthreads();
     fold_candidate(s, C, kb, i);
-    if (threadIdx.x == 0) C.stats[S_ACC] += 1;
+    if (threadIdx.x == 0) {
+      C.stats[S_ACC] += 1;
+      if (i > 0) s.clean[i - 1] = 0;
+      s.clean[i + 1] = 0;
+    }
     ++*accepted;
   }
   prof_lap(C, P_APPLYQ, tp);
-  const int bb = C.bond_bound[i + 1];
-  const int cap = e.chi_max < bb ? e.chi_max : bb;
   // Nothing applied and the identity class's Gram has exactly chi eigenvalues above
   // max(1e-12, 4 cutoff^2) tr (theta has rank <= chi, the bond dimension): every one of those
   // Schmidt values is above 1e-6 s_0 and above the cutoff, so the truncated SVD would keep the bond
   // as it is.  A QR move of the centre gives the same state and bond dimension without it.
-  const int chim = C.dims[i + 1];
   if (kb == 0 && s.rank0 == chim && chim <= cap) {
     if (big) {   // release the other CTAs
       if (threadIdx.x == 0) s.jmode = 0;
@@ -3003,12 +3212,10 @@ __device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, i
     if (ltr) move_right(s, C, i);
     else move_left_qr(s, C, i + 1);
     note_chi(C, chim);
+    if (threadIdx.x == 0) s.clean[i] = 1;
     __syncthreads();
     prof_lap(C, P_QRMOVE, tp);
-    if (prof_thread(C)) {
-      C.prof[P_VCYC + prof_bucket(m)] += clock64() - tv;
-      C.prof[P_CURB] = 0;
-    }
+    end_visit(C, m, tv);
     return;
   }
   Factor F;
@@ -3050,55 +3257,64 @@ __device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, i
     C.dims[i + 1] = k;
     C.meta[M_OC] = ltr ? i + 1 : i;
     C.dstats[0] += F.disc;
+    // the certificate of a QR move, from the (unit norm) singular values themselves; a truncation that moves the
+    // state by more than rounding can change the scores at every bond
+    const double sk = C.sing[k - 1];
+    s.clean[i] = F.disc <= 1e-24 && sk * sk > fmax(1e-12, 4.0 * e.cutoff * e.cutoff);
   }
+  if (F.disc > 1e-24)
+    for (int b = threadIdx.x; b < C.n; b += blockDim.x)
+      if (b != i) s.clean[b] = 0;
   note_chi(C, k);
   __syncthreads();
   prof_lap(C, P_SPLIT, tp);
-  if (prof_thread(C)) {
-    C.prof[P_VCYC + prof_bucket(m)] += clock64() - tv;
-    C.prof[P_CURB] = 0;
-  }
+  end_visit(C, m, tv);
 }
 
-// Alternating sweeps over the bonds of the last span; every CTA of the cluster runs the loop, only
-// the leader touches the MPS and the tableau.
+// Alternating sweeps over the bonds of the last span: the leader runs them, the other CTAs serve its visits.
 // sweep_cap > 0 overrides the handle's max_sweeps for this call; visit_cap > 0 stops after that
 // many bond visits (the centre is then left where the last split put it).
 __device__ void disentangle(Smem& s, Smem* lead, const Ctx& C, int sweep_cap, int visit_cap) {
-  cluster_sync();
-  if (C.meta[M_STATUS] != 0) return;   // a failed circuit does no further work
-  if (!C.meta[M_HAVE_SPAN]) return;
-  const int f = C.meta[M_F], l = C.meta[M_L];
-  if (l <= f) return;
-  const int max_sweeps = sweep_cap > 0 ? sweep_cap : C.e->max_sweeps;
-  int visits = 0;
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    const bool ltr = (sweep & 1) == 0;
-    long long tp = prof_start(C);
-    if (C.rank == 0) move_center(s, C, ltr ? f : l);
-    prof_lap(C, P_CENTER, tp);
-    int acc = 0;
-    bool capped = false;
-    for (int t = 0; t < l - f; ++t) {
-      if (visit_cap > 0 && visits >= visit_cap) {
-        capped = true;
-        break;
-      }
-      const int i = ltr ? f + t : l - 1 - t;
-      visit_bond(s, lead, C, i, ltr, &acc);
-      ++visits;
-    }
-    if (capped) break;
-    if (C.rank == 0 && threadIdx.x == 0) {
-      C.stats[S_SWEEPS] += 1;
-      s.bcast = acc;
-    }
-    cluster_sync();
-    const int acc_all = lead->bcast;
-    const int failed = C.meta[M_STATUS];
-    cluster_sync();   // every CTA has read bcast and the status before either changes
-    if (acc_all == 0 || failed != 0) break;
+  cluster_sync();   // every CTA has left the sweeps of the previous call before vbond changes
+  if (C.rank != 0) {
+    serve_visits(s, lead, C);
+    return;
   }
+  const int f = C.meta[M_F], l = C.meta[M_L];
+  const int max_sweeps = sweep_cap > 0 ? sweep_cap : C.e->max_sweeps;
+  // a failed circuit does no further work
+  if (C.meta[M_STATUS] == 0 && C.meta[M_HAVE_SPAN] && l > f) {
+    for (int b = threadIdx.x; b < C.n; b += blockDim.x) s.clean[b] = 0;
+    __syncthreads();
+    int visits = 0;
+    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
+      const bool ltr = (sweep & 1) == 0;
+      long long tp = prof_start(C);
+      move_center(s, C, ltr ? f : l);
+      prof_lap(C, P_CENTER, tp);
+      int acc = 0;
+      bool capped = false;
+      for (int t = 0; t < l - f; ++t) {
+        if (visit_cap > 0 && visits >= visit_cap) {
+          capped = true;
+          break;
+        }
+        const int i = ltr ? f + t : l - 1 - t;
+        const bool last = (t == l - f - 1 && (acc == 0 || sweep + 1 == max_sweeps)) ||
+                          (visit_cap > 0 && visits + 1 >= visit_cap);
+        visit_bond(s, lead, C, i, ltr, last, &acc);
+        ++visits;
+      }
+      if (capped) break;
+      if (threadIdx.x == 0) C.stats[S_SWEEPS] += 1;
+      const int failed = C.meta[M_STATUS];
+      __syncthreads();
+      if (acc == 0 || failed != 0) break;
+    }
+  }
+  if (threadIdx.x == 0) s.vbond = -1;
+  __syncthreads();
+  cluster_sync();
 }
 
 __device__ void init_tau(Smem& s, int d) {
@@ -3186,13 +3402,15 @@ __device__ __forceinline__ void run_body(const Engine& e, const gcamps_op* ops, 
   Ctx C = make_ctx(e, c, rank);
   Smem* lead = cg::this_cluster().map_shared_rank(&s, 0);
   init_tau(s, e.d);
-  if (C.prof && threadIdx.x == 0 && rank < kProfSmids) {   // where the cluster's CTAs run (1 + SM id)
+  load_counters(s, C);
+  if (threadIdx.x == 0 && rank < kProfSmids) {   // where the cluster's CTAs run (1 + SM id)
     unsigned sm;
     asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
-    C.prof[P_SMID + rank] = 1 + (long long)sm;
+    e.prof[(long long)c * P_COUNT + P_SMID + rank] = 1 + (long long)sm;
   }
   if (GCAMPS_TC && e.tc_smem) tc_setup(s);
   for (int i = first; i < stop; ++i) run_op(s, lead, C, ops[i]);
+  store_counters(s, C);
   cluster_sync();
   if (GCAMPS_TC && e.tc_smem) tc_teardown(s);
 }
@@ -3204,7 +3422,9 @@ __device__ __forceinline__ void single_body(const Engine& e, const gcamps_op& op
   Smem* lead = cg::this_cluster().map_shared_rank(&s, 0);
   init_tau(s, e.d);
   if (GCAMPS_TC && e.tc_smem) tc_setup(s);
+  load_counters(s, C);
   run_op(s, lead, C, op);
+  store_counters(s, C);
   cluster_sync();
   if (GCAMPS_TC && e.tc_smem) tc_teardown(s);
 }
@@ -3232,7 +3452,7 @@ __device__ __forceinline__ void score_theta_body(const Engine& e, const double2*
     }
   cluster_sync();
   int nev = 0;
-  const int kb = select_class(s, lead, C, th, cl, cr, &nev);
+  const int kb = select_class(s, lead, C, th, cl, cr, &nev, false);
   if (c == 0 && rank == 0 && threadIdx.x == 0) {
     out_choice[0] = kb;
     out_choice[1] = nev;

@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) k_score_theta_static(Engin
     }
   cluster_sync();
   int nev = 0;
-  const int kb = select_class(s, lead, C, th, cl, cr, &nev);
+  const int kb = select_class(s, lead, C, th, cl, cr, &nev, false);
   cluster_sync();
   if (rank == 0 && threadIdx.x == 0) {
     out_choice[0] = kb;
