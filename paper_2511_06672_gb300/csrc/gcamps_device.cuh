@@ -44,6 +44,10 @@ namespace cg = cooperative_groups;
 constexpr int kPruneMin = 1;
 // CTA-level eigenvalue multisection keeps the tridiagonal in shared memory up to this size.
 constexpr int kBTri = 256;
+// Small factorisations keep their matrix in shared memory (svd_small, qr_small): at most this many entries, and
+// fewer than kClusterJacobiMin columns.
+constexpr int kZ = 1024;
+constexpr int kZCols = kClusterJacobiMin;
 
 // (i, j), j <= i, of entry t of the row-major packed lower triangle (t = i (i + 1) / 2 + j).
 __device__ __forceinline__ void tri_index(int t, int& i, int& j) {
@@ -134,6 +138,52 @@ __device__ __forceinline__ int warp_sum_int(int v) {
   return v;
 }
 
+// The same over aligned groups of G lanes (a power of two, 4 <= G <= 32; the whole warp calls it).
+__device__ __forceinline__ void group_sum4(double& a, double& b, double& c, double& d, int G) {
+  const int lane = threadIdx.x & 31;
+  const bool h1 = lane & (G >> 1), h2 = lane & (G >> 2);
+  double k0 = h1 ? c : a, k1 = h1 ? d : b;
+  k0 += __shfl_xor_sync(0xffffffffu, h1 ? a : c, G >> 1);
+  k1 += __shfl_xor_sync(0xffffffffu, h1 ? b : d, G >> 1);
+  double v = h2 ? k1 : k0;
+  v += __shfl_xor_sync(0xffffffffu, h2 ? k0 : k1, G >> 2);
+  for (int o = G >> 3; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  const int base = lane & ~(G - 1);
+  a = __shfl_sync(0xffffffffu, v, base);
+  b = __shfl_sync(0xffffffffu, v, base + (G >> 2));
+  c = __shfl_sync(0xffffffffu, v, base + (G >> 1));
+  d = __shfl_sync(0xffffffffu, v, base + 3 * (G >> 2));
+}
+__device__ __forceinline__ void group_sum2(double& a, double& b, int G) {
+  const int lane = threadIdx.x & 31;
+  const bool h = lane & (G >> 1);
+  double v = h ? b : a;
+  v += __shfl_xor_sync(0xffffffffu, h ? a : b, G >> 1);
+  for (int o = G >> 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  const int base = lane & ~(G - 1);
+  a = __shfl_sync(0xffffffffu, v, base);
+  b = __shfl_sync(0xffffffffu, v, base + (G >> 1));
+}
+// Lanes that share a column of m entries: one pass over it where it fits a warp.
+__device__ __forceinline__ int lanes_for(int m) { return m <= 8 ? 8 : (m <= 16 ? 16 : 32); }
+
+// 1 / sqrt(a) for a in the normal range: the hardware's approximation y and one step of the cubically convergent
+// iteration y (1 + e/2 + 3 e^2/8), e = 1 - a y^2: five FP64 instructions of 64 cycles.  The first step's error
+// 5 e^3 / 16 is below 2^-56 for an approximation good to 2^-18.
+__device__ __forceinline__ double rsqrt_fast(double a) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double e = fma(-(a * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+// 1 / a for a in the normal range, by y (1 + e + e^2), e = 1 - a y.
+__device__ __forceinline__ double rcp_fast(double a) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double e = fma(-a, y, 1.0);
+  return fma(y * e, 1.0 + e, y);
+}
+
 // -------------------------------------------------------------------------- per-CTA workspace
 struct Smem {
   uint8_t lut[81 * 5];        // conjugation table of the current two-qudit Clifford
@@ -153,16 +203,23 @@ struct Smem {
   double vbd[kMaxK];          // its error bound: |vest - S_vN| <= vbd (cluster leader)
   uint8_t estd[kMaxK];        // vest[k] valid
   int rk[kMaxK];              // weight rank of each exactly evaluated class (cluster leader)
-  double wtri[kWarps][64];    // per warp: tridiagonal diagonal [0, 32) | off-diagonal squared [32, 64)
-  float wtri32[kWarps][64];   // the same in FP32
-  double btri[2 * kBTri];     // CTA-level: diagonal | off-diagonal squared
-  float btri32[2 * kBTri];
-  float2 hv[kBTri], hw[kBTri];  // FP32 Householder reduction: reflector v and w = p - K v of the current column
-  // the second half-CTA group's copies (two FP32 estimates at once, HalfGroup) and both halves' partial sums
-  float2 hv2[kBTri], hw2[kBTri];
-  float btri32b[2 * kBTri];
-  float redh[2][kWarps / 2];
-  float2 whv[kWarps][32], whw[kWarps][32];   // the same per warp (warp-level estimates, m <= 32)
+  // Scoring and the small factorisations never overlap on a CTA (a cluster barrier lies between): they share the
+  // space, which leaves the SM's L1 to the scratch in global memory.
+  union {
+    struct {
+      double wtri[kWarps][64];    // per warp: tridiagonal diagonal [0, 32) | off-diagonal squared [32, 64)
+      float wtri32[kWarps][64];   // the same in FP32
+      double btri[2 * kBTri];     // CTA-level: diagonal | off-diagonal squared
+      float btri32[2 * kBTri];
+      float2 hv[kBTri], hw[kBTri];  // FP32 Householder reduction: reflector v and w = p - K v of the current column
+      // the second half-CTA group's copies (two FP32 estimates at once, HalfGroup)
+      float2 hv2[kBTri], hw2[kBTri];
+      float btri32b[2 * kBTri];
+      float2 whv[kWarps][32], whw[kWarps][32];   // the same per warp (warp-level estimates, m <= 32)
+    };
+    double2 z[kZ];              // small factorisations: the matrix, column by column
+  };
+  float redh[2][kWarps / 2];    // partial sums of the half-CTA groups
   int jmode, jm, jn;          // cluster split of a bond visit: 0 none, 2 cluster Jacobi; its matrix shape (leader)
   int jflag[2];               // cluster Jacobi: a rotation happened in the sweep of this parity (leader)
   double jfro;                // cluster Jacobi: |B|_F^2 (leader)
@@ -176,6 +233,10 @@ struct Smem {
   uint64_t tc_mbar;           // tensor-core Gram: completion barrier of its MMAs
   uint32_t tc_tmem;           // its TMEM accumulator (column base)
   uint32_t tc_commits;        // commits on tc_mbar so far (its phase parity)
+  double zs[kZCols], zinv[kZCols];   // singular values of z in order (times the scale), and their inverses
+  double2 zdiag[kZCols];      // QR: diagonal of R
+  double zbeta[kZCols];       // QR: reflector scalars
+  int zperm[kZCols];
   int npure, pure;            // select_class: classes of the purity test, and whether it decided (leader)
   int vbond;                  // bond of the visit the cluster serves next, -1 to leave the sweeps (leader)
   uint8_t clean[kMaxN];       // bond b: the state around it is the one its last visit left (leader, disentangle)
@@ -830,11 +891,327 @@ __device__ __noinline__ Factor svd_finish(Smem& s, const Ctx& C, const SvdPrep& 
   return F;
 }
 
+// ------------------------------------------------------------ small factorisations in shared memory
+// Up to a few hundred entries a factorisation is bound by its chain of FP64 instructions (64 cycles of a
+// sub-partition's pipe for a warp's instruction, whatever its active lanes), not by their number: these routines
+// keep the matrix in shared memory, give a column (pair) just the lanes it fills, put the groups on different
+// pipes, and cut the instructions of each link.
+__device__ __forceinline__ bool svd_fits(int rows, int cols) {
+  const int n = rows < cols ? rows : cols, m = rows < cols ? cols : rows;
+  return n < kZCols && n * (m + n) <= kZ;
+}
+
+// The rotations of jacobi_orthogonalize on the columns of s.z, each the m entries of B over the n of W (stride m + n),
+// so that one pass rotates both.  Rounds: for odd n the pairs with i + j = 2 round (mod n), (n - 1) / 2 of them and
+// no idle slot; for even n the round-robin of jacobi_orthogonalize.  The rotation's cosine and sine come from two
+// reciprocal square roots: with r = 1 / sqrt(1 + zeta^2), c^2 = (1 + |zeta| r) / 2 and s c = r / 2.  About 40 FP64
+// instructions a pair instead of 130; a 9-column sweep takes 30 instead of 90 kcycles.  n = 2, 3 has one pair a
+// round: one warp does it without CTA barriers.
+__device__ int jacobi_small(Smem& s, int m, int n, double fro, int max_sweeps) {
+  if (n <= 1) return 0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int L = m + n, G = lanes_for(L), P = 32 / G;
+  const int npairs = n / 2, rounds = n - 1 + (n & 1);
+  const bool one = npairs == 1;
+  const long long zc_bits = __double_as_longlong(1e-30 * fro);
+  const double tol2 = 1e-28;
+  const int sub = lane / G, r0 = lane & (G - 1);
+  int sweeps = -1;
+  for (int sweep = 0; sweep < max_sweeps && !(one && warp > 0); ++sweep) {
+    bool any = false;
+    for (int round = 0; round < rounds; ++round) {
+      for (int p0 = warp; p0 < npairs; p0 += kWarps * P) {
+        const int p = p0 + kWarps * sub;
+        const bool act = p < npairs;
+        int i = 0, j = 0;
+        if (act) {
+          if (n & 1) {
+            i = round + p + 1;
+            j = round - p - 1;
+            if (i >= n) i -= n;
+            if (j < 0) j += n;
+          } else {
+            i = (p == 0) ? 0 : 1 + ((p - 1 + round) % (n - 1));
+            j = 1 + ((n - 2 - p + round) % (n - 1));
+          }
+          if (i > j) {
+            const int t = i;
+            i = j;
+            j = t;
+          }
+        }
+        double2* bi = s.z + i * L;
+        double2* bj = s.z + j * L;
+        double al = 0, be = 0, gr = 0, gi = 0;
+        if (act)
+          for (int r = r0; r < m; r += G) {
+            const double2 x = bi[r], y = bj[r];
+            al = fma(x.x, x.x, fma(x.y, x.y, al));
+            be = fma(y.x, y.x, fma(y.y, y.y, be));
+            gr = fma(x.x, y.x, fma(x.y, y.y, gr));
+            gi = fma(x.x, y.y, fma(-x.y, y.x, gi));
+          }
+        group_sum4(al, be, gr, gi, G);
+        if (!act || __double_as_longlong(al) <= zc_bits || __double_as_longlong(be) <= zc_bits) continue;
+        const double g2 = fma(gr, gr, gi * gi);
+        if (!(g2 > tol2 * al * be) || g2 < 1e-290) continue;
+        const double ig = rsqrt_fast(g2);
+        const double zeta = (be - al) * (0.5 * ig);
+        const double r = rsqrt_fast(fma(zeta, zeta, 1.0));
+        const double c2 = fma(0.5 * fabs(zeta), r, 0.5);
+        const double q = rsqrt_fast(c2);
+        const double cs = c2 * q, sn = copysign(0.5 * r * q, zeta) * ig;
+        const double a = gr * sn, b = gi * sn;   // s gamma / |gamma|
+        for (int t = r0; t < L; t += G) {
+          const double2 x = bi[t], y = bj[t];
+          bi[t] = make_double2(fma(cs, x.x, fma(-a, y.x, -b * y.y)), fma(cs, x.y, fma(-a, y.y, b * y.x)));
+          bj[t] = make_double2(fma(cs, y.x, fma(a, x.x, -b * x.y)), fma(cs, y.y, fma(a, x.y, b * x.x)));
+        }
+        any = true;
+      }
+      if (one) __syncwarp();
+      else __syncthreads();
+    }
+    const bool rotated = one ? __any_sync(0xffffffffu, any) : __syncthreads_or(any);
+    if (!rotated) {
+      sweeps = sweep + 1;
+      break;
+    }
+  }
+  if (one) {
+    if (threadIdx.x == 0) s.ival[3] = sweeps;
+    __syncthreads();
+    sweeps = s.ival[3];
+  }
+  return sweeps;
+}
+
+// Truncated SVD of M (rows x cols, row-major; svd_fits) with svd_factor's rules, written where the caller wants it:
+// U (rows x k), times the kept singular values if us, and Vh (k x cols), times them if vs.  M may be U or Vh.  Sizes
+// that svd_factor first reduces by a QR go without: the rows that saves cost nothing here.  C.sing as svd_factor's.
+struct SmallSplit {
+  int k;
+  double disc;
+};
+__device__ __noinline__ SmallSplit svd_small(Smem& s, const Ctx& C, const double2* M, int rows, int cols, int cap,
+                                             bool renorm, double2* U, bool us, double2* Vh, bool vs) {
+  const Engine& e = *C.e;
+  const bool tall = rows >= cols;
+  const int m = tall ? rows : cols, n = tall ? cols : rows, L = m + n;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double fro = 0;
+  for (int idx = threadIdx.x; idx < rows * cols; idx += blockDim.x) {
+    const int r = idx / cols, c = idx % cols;
+    const double2 v = M[idx];
+    fro = fma(v.x, v.x, fma(v.y, v.y, fro));
+    if (tall) s.z[c * L + r] = v;
+    else s.z[r * L + c] = cconj(v);
+  }
+  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x)
+    s.z[(idx / n) * L + m + idx % n] = make_double2(idx / n == idx % n ? 1.0 : 0.0, 0.0);
+  fro = block_sum(fro, s);
+  const int sweeps = jacobi_small(s, m, n, fro, e.jacobi_cap);
+  // column norms, G lanes a column
+  const int G = lanes_for(m), P = 32 / G;
+  for (int j0 = warp; j0 < n; j0 += kWarps * P) {
+    const int j = j0 + kWarps * (lane / G);
+    double a = 0, b = 0;
+    if (j < n)
+      for (int r = lane & (G - 1); r < m; r += G) a += cabs2(s.z[j * L + r]);
+    group_sum2(a, b, G);
+    if (j < n && (lane & (G - 1)) == 0) s.zinv[j] = a;
+  }
+  __syncthreads();
+  // order, rank rule and scale on the first warp, a lane per column
+  if (warp == 0) {
+    const double v2 = lane < n ? s.zinv[lane] : 0.0;
+    const long long key = __double_as_longlong(v2);   // >= 0: ordered as integers
+    int rank = 0;
+    for (int i = 0; i < n; ++i) {
+      const long long ki = __shfl_sync(0xffffffffu, key, i);
+      rank += (ki > key) || (ki == key && i < lane);
+    }
+    const double v = lane < n ? sqrt(v2) : 0.0;
+    __syncwarp();
+    if (lane < n) {
+      s.zperm[rank] = lane;
+      s.zs[rank] = v;
+    }
+    __syncwarp();
+    const double sv = lane < n ? s.zs[lane] : 0.0;
+    const double s0 = __shfl_sync(0xffffffffu, sv, 0);
+    int k = __popc(__ballot_sync(0xffffffffu, lane < n && s0 > 0.0 && sv > e.cutoff * s0));
+    if (k > cap) k = cap;
+    if (k < 1) k = 1;
+    double kept = lane < k ? sv * sv : 0.0, drop = lane < k ? 0.0 : sv * sv;
+    group_sum2(kept, drop, 32);
+    const double scale = (renorm && kept > 0) ? 1.0 / sqrt(kept) : 1.0;
+    if (lane < n) {
+      s.zinv[lane] = sv > 0.0 ? 1.0 / sv : 0.0;
+      s.zs[lane] = sv * scale;
+      C.sing[lane] = lane < k ? sv * scale : sv;
+    }
+    if (lane == 0) {
+      s.ival[0] = k;
+      s.dval[0] = drop;
+      s.dval[1] = scale;
+      if (sweeps < 0) set_failure(C, GCAMPS_ENOCONV, 1, rows, cols);
+      const int sw = sweeps < 0 ? e.jacobi_cap : sweeps;
+      C.stats[S_SVD] += 1;
+      C.stats[S_JSWEEPS] += sw;
+      if (sw > C.stats[S_JMAX]) C.stats[S_JMAX] = sw;
+    }
+  }
+  __syncthreads();
+  const int k = s.ival[0];
+  const double scale = s.dval[1];
+  for (int idx = threadIdx.x; idx < rows * k; idx += blockDim.x) {
+    const int r = idx / k, i = idx % k;
+    const double2* col = s.z + s.zperm[i] * L;
+    U[idx] = tall ? cscale(col[r], us ? scale : s.zinv[i]) : (us ? cscale(col[m + r], s.zs[i]) : col[m + r]);
+  }
+  for (int idx = threadIdx.x; idx < k * cols; idx += blockDim.x) {
+    const int i = idx / cols, c = idx % cols;
+    const double2* col = s.z + s.zperm[i] * L;
+    const double2 v = cconj(tall ? col[m + c] : col[c]);
+    Vh[idx] = tall ? (vs ? cscale(v, s.zs[i]) : v) : cscale(v, vs ? scale : s.zinv[i]);
+  }
+  SmallSplit f;
+  f.k = k;
+  f.disc = s.dval[0];
+  __syncthreads();
+  return f;
+}
+
+// Householder QR of the m x n matrix in s.z (column-major, stride m; m n + m min(m, n) <= kZ, n < kZCols) with
+// block_qr's reflectors: R's part above the diagonal stays in s.z, its diagonal goes to s.zdiag, Q (m x k) follows
+// the matrix.  One barrier a step: the group that owns the next column takes that column's norm and reflector
+// right after its update, the other columns' groups meanwhile finish theirs; Q's columns need none (column c is
+// H_0 .. H_c e_c).  9 x 3: 12 instead of 25 kcycles.
+__device__ __forceinline__ bool qr_fits(int m, int n) { return n < kZCols && m * n + m * (m < n ? m : n) <= kZ; }
+
+__device__ int qr_small(Smem& s, int m, int n, double fro) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int k = m < n ? m : n;
+  const int G = lanes_for(m), P = 32 / G, sub = lane / G, r0 = lane & (G - 1);
+  const double tiny = 1e-30 * fro;
+  // column c belongs to group c % (kWarps P): warp c % kWarps, its part (c / kWarps) % P
+  auto reflector = [&](int j, bool act) {   // the warp's group `act` makes column j's reflector
+    double2* x = s.z + j * m;
+    double nrm2 = 0, dummy = 0;
+    if (act)
+      for (int r = r0; r < m; r += G)
+        if (r >= j) nrm2 += cabs2(x[r]);
+    group_sum2(nrm2, dummy, G);
+    if (!act || r0 != 0) return;
+    const double2 x0 = x[j];
+    if (nrm2 <= tiny) {
+      s.zbeta[j] = 0.0;
+      s.zdiag[j] = x0;
+      return;
+    }
+    const double s0 = fma(x0.x, x0.x, x0.y * x0.y);
+    const bool fast = s0 > 0x1p-900 && s0 < 0x1p+900;
+    const double rs = fast ? rsqrt_fast(s0) : 0.0;
+    const double ax0 = fast ? s0 * rs : hypot(x0.x, x0.y);
+    const double2 ph = fast ? make_double2(x0.x * rs, x0.y * rs) : unit_phase(x0);
+    const bool norm = nrm2 > 0x1p-900 && nrm2 < 0x1p+900;
+    const double alpha = norm ? nrm2 * rsqrt_fast(nrm2) : sqrt(nrm2);
+    const double h = alpha * (alpha + ax0);
+    s.zbeta[j] = norm ? rcp_fast(h) : 1.0 / h;
+    x[j] = make_double2(fma(ph.x, alpha, x0.x), fma(ph.y, alpha, x0.y));
+    s.zdiag[j] = make_double2(-ph.x * alpha, -ph.y * alpha);
+  };
+  // y -= beta v (v^H y) on rows j.. for the group's column y
+  auto reflect = [&](const double2* v, double bt, int j, double2* y, bool act) {
+    double wr = 0, wi = 0;
+    if (act)
+      for (int r = r0; r < m; r += G)
+        if (r >= j) {
+          const double2 x = v[r], t = y[r];
+          wr = fma(x.x, t.x, fma(x.y, t.y, wr));
+          wi = fma(x.x, t.y, fma(-x.y, t.x, wi));
+        }
+    group_sum2(wr, wi, G);
+    if (!act) return;
+    wr *= bt;
+    wi *= bt;
+    for (int r = r0; r < m; r += G)
+      if (r >= j) {
+        const double2 x = v[r];
+        double2 t = y[r];
+        t.x = fma(-x.x, wr, fma(x.y, wi, t.x));
+        t.y = fma(-x.x, wi, fma(-x.y, wr, t.y));
+        y[r] = t;
+      }
+  };
+  if (warp == 0) reflector(0, sub == 0);
+  __syncthreads();
+  for (int j = 0; j < k; ++j) {
+    const double bt = s.zbeta[j];
+    for (int c0 = warp; c0 < n; c0 += kWarps * P) {
+      if (c0 + kWarps * (P - 1) <= j) continue;   // all of the warp's columns are done
+      const int c = c0 + kWarps * sub;
+      const bool act = c > j && c < n;
+      if (bt != 0.0) reflect(s.z + j * m, bt, j, s.z + c * m, act);
+      const int nx = j + 1;
+      if (nx < k && nx % kWarps == warp && nx >= c0 && nx < c0 + kWarps * P) {
+        __syncwarp();
+        reflector(nx, c == nx);
+      }
+    }
+    __syncthreads();
+  }
+  // Q
+  double2* Q = s.z + m * n;
+  for (int c0 = warp; c0 < k; c0 += kWarps * P) {
+    const int c = c0 + kWarps * sub;
+    const bool own = c < k;
+    if (own)
+      for (int r = r0; r < m; r += G) Q[c * m + r] = make_double2(r == c ? 1.0 : 0.0, 0.0);
+    __syncwarp();
+    const int top = min(c0 + kWarps * (P - 1), k - 1);
+    for (int j = top; j >= 0; --j) {
+      const double bt = s.zbeta[j];
+      if (bt != 0.0) reflect(s.z + j * m, bt, j, Q + c * m, own && j <= c);
+    }
+  }
+  __syncthreads();
+  return k;
+}
+// Entry (i, c) of qr_small's R.
+__device__ __forceinline__ double2 small_r(const Smem& s, int m, int i, int c) {
+  return c > i ? s.z[c * m + i] : (c == i ? s.zdiag[i] : cz());
+}
+
+// out <- f(0..count-1) where f reads out's old entries: each thread keeps its results until every thread has read.
+constexpr int kStaged = 4 * kThreads;
+template <class F>
+__device__ __forceinline__ void staged(double2* out, int count, F f) {
+  double2 v[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+    if (threadIdx.x + t * kThreads < count) v[t] = f(threadIdx.x + t * kThreads);
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+    if (threadIdx.x + t * kThreads < count) out[threadIdx.x + t * kThreads] = v[t];
+}
+
 // Factor M (rows x cols, row-major) = U S Vh keeping the k largest singular values with
 // s_i > cutoff * s_0 (at most cap, at least one), on this CTA alone.
 __device__ __noinline__ Factor svd_factor(Smem& s, const Ctx& C, const double2* M, int rows, int cols, int cap,
                                           bool renorm) {
   const Engine& e = *C.e;
+  if (svd_fits(rows, cols)) {
+    Factor F;
+    F.U = C.scr + e.sl.u;
+    F.Vh = C.scr + e.sl.vh;
+    const SmallSplit f = svd_small(s, C, M, rows, cols, cap, renorm, F.U, false, F.Vh, false);
+    F.k = f.k;
+    F.disc = f.disc;
+    return F;
+  }
   const SvdPrep p = svd_prepare(s, C, M, rows, cols);
   const int sweeps = jacobi_orthogonalize(s, C.scr + e.sl.b, p.mm, p.n, C.scr + e.sl.w, e.jacobi_cap);
   return svd_finish(s, C, p, sweeps, rows, cols, cap, renorm);
@@ -973,11 +1350,35 @@ __device__ void move_right(Smem& s, const Ctx& C, int j) {
     move_unit(s, C, A, cl * d, A2, d * cr2, j + 1);
     return;
   }
+  const int m = cl * d, n = cr;
+  if (qr_fits(m, n) && min(m, n) * d * cr2 <= kStaged) {
+    double fro = 0;
+    for (int idx = threadIdx.x; idx < m * n; idx += blockDim.x) {
+      const double2 v = A[idx];
+      fro = fma(v.x, v.x, fma(v.y, v.y, fro));
+      s.z[(idx % n) * m + idx / n] = v;
+    }
+    fro = block_sum(fro, s);
+    const int k = qr_small(s, m, n, fro), w = d * cr2;
+    for (int idx = threadIdx.x; idx < m * k; idx += blockDim.x) A[idx] = s.z[m * n + (idx % k) * m + idx / k];
+    staged(A2, k * w, [&](int idx) {
+      const int i = idx / w, col = idx % w;
+      double2 acc = cz();
+      for (int c = i; c < n; ++c) acc = cfma(small_r(s, m, i, c), A2[c * w + col], acc);
+      return acc;
+    });
+    if (threadIdx.x == 0) {
+      C.stats[S_QR] += 1;
+      C.dims[j + 1] = k;
+      C.meta[M_OC] = j + 1;
+    }
+    __syncthreads();
+    return;
+  }
   double2* B = C.scr + e.sl.b;
   double2* Q = C.scr + e.sl.u;
   double2* R = C.scr + e.sl.vh;
   double2* tmp = C.scr + e.sl.tmp;
-  const int m = cl * d, n = cr;
   for (long long idx = threadIdx.x; idx < (long long)m * n; idx += blockDim.x) {
     const int r = (int)(idx / n), c = (int)(idx % n);
     B[(long long)c * m + r] = A[idx];
@@ -1012,12 +1413,36 @@ __device__ void move_left_qr(Smem& s, const Ctx& C, int j) {
     move_unit(s, C, A, d * cr, A0, cl2 * d, j - 1);
     return;
   }
+  const int m = d * cr, n = cl;   // M^H is m x n
+  if (qr_fits(m, n) && cl2 * d * min(m, n) <= kStaged) {
+    double fro = 0;
+    for (int idx = threadIdx.x; idx < n * m; idx += blockDim.x) {
+      const double2 v = A[idx];
+      fro = fma(v.x, v.x, fma(v.y, v.y, fro));
+      s.z[idx] = cconj(v);
+    }
+    fro = block_sum(fro, s);
+    const int k = qr_small(s, m, n, fro);
+    for (int idx = threadIdx.x; idx < k * m; idx += blockDim.x) A[idx] = cconj(s.z[m * n + idx]);
+    staged(A0, cl2 * d * k, [&](int idx) {
+      const int r = idx / k, i = idx % k;
+      double2 acc = cz();
+      for (int c = i; c < n; ++c) acc = cfmac(small_r(s, m, i, c), A0[r * n + c], acc);
+      return acc;
+    });
+    if (threadIdx.x == 0) {
+      C.stats[S_QR] += 1;
+      C.dims[j] = k;
+      C.meta[M_OC] = j - 1;
+    }
+    __syncthreads();
+    return;
+  }
   double2* B = C.scr + e.sl.b;
   double2* Q = C.scr + e.sl.u;
   double2* R = C.scr + e.sl.vh;
   double2* tmp = C.scr + e.sl.tmp;
   double2* RH = C.scr + e.sl.w;
-  const int m = d * cr, n = cl;   // M^H is m x n
   for (long long idx = threadIdx.x; idx < (long long)n * m; idx += blockDim.x) {
     const int a = (int)(idx / m), c = (int)(idx % m);      // M[a][c]
     B[(long long)a * m + c] = cconj(A[idx]);
@@ -1086,6 +1511,23 @@ __device__ double move_left(Smem& s, const Ctx& C, int j, int cap, bool renorm, 
   double2* A = site_ptr(C, j);
   double2* A0 = site_ptr(C, j - 1);
   const int bb = C.bond_bound[j];
+  if (svd_fits(cl, d * cr) && cl2 * d * min(cl, d * cr) <= kStaged) {
+    double2* US = C.scr + C.e->sl.u;
+    const SmallSplit f = svd_small(s, C, A, cl, d * cr, cap < bb ? cap : bb, renorm, US, true, A, false);
+    const int k = f.k;
+    staged(A0, cl2 * d * k, [&](int idx) {
+      const int r = idx / k, i = idx % k;
+      double2 acc = cz();
+      for (int c = 0; c < cl; ++c) acc = cfma(A0[r * cl + c], US[c * k + i], acc);
+      return acc;
+    });
+    if (threadIdx.x == 0) {
+      C.dims[j] = k;
+      C.meta[M_OC] = j - 1;
+    }
+    __syncthreads();
+    return f.disc;
+  }
   Factor F = lead ? svd_factor_cluster(s, lead, C, A, cl, d * cr, cap < bb ? cap : bb, renorm)
                   : svd_factor(s, C, A, cl, d * cr, cap < bb ? cap : bb, renorm);
   const int k = F.k;
@@ -3219,7 +3661,11 @@ __device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, b
     return;
   }
   Factor F;
-  if (big) {
+  if (svd_fits(rows, cols)) {
+    const SmallSplit f = svd_small(s, C, theta, rows, cols, cap, true, site_ptr(C, i), !ltr, site_ptr(C, i + 1), ltr);
+    F.k = f.k;
+    F.disc = f.disc;
+  } else if (big) {
     const SvdPrep p = svd_prepare(s, C, theta, rows, cols);
     double2* B = C.scr + e.sl.b;
     double2* W = C.scr + e.sl.w;
@@ -3243,16 +3689,18 @@ __device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, b
     F = svd_factor(s, C, theta, rows, cols, cap, true);
   }
   const int k = F.k;
-  if (ltr) {
-    for (long long idx = threadIdx.x; idx < (long long)k * d * cr; idx += blockDim.x)
-      F.Vh[idx] = cscale(F.Vh[idx], C.sing[idx / (d * cr)]);
-  } else {
-    for (long long idx = threadIdx.x; idx < (long long)cl * d * k; idx += blockDim.x)
-      F.U[idx] = cscale(F.U[idx], C.sing[idx % k]);
+  if (!svd_fits(rows, cols)) {
+    if (ltr) {
+      for (long long idx = threadIdx.x; idx < (long long)k * d * cr; idx += blockDim.x)
+        F.Vh[idx] = cscale(F.Vh[idx], C.sing[idx / (d * cr)]);
+    } else {
+      for (long long idx = threadIdx.x; idx < (long long)cl * d * k; idx += blockDim.x)
+        F.U[idx] = cscale(F.U[idx], C.sing[idx % k]);
+    }
+    __syncthreads();
+    block_copy(site_ptr(C, i), F.U, (long long)cl * d * k);
+    block_copy(site_ptr(C, i + 1), F.Vh, (long long)k * d * cr);
   }
-  __syncthreads();
-  block_copy(site_ptr(C, i), F.U, (long long)cl * d * k);
-  block_copy(site_ptr(C, i + 1), F.Vh, (long long)k * d * cr);
   if (threadIdx.x == 0) {
     C.dims[i + 1] = k;
     C.meta[M_OC] = ltr ? i + 1 : i;
