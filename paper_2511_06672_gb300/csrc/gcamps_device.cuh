@@ -185,12 +185,15 @@ __device__ __forceinline__ double rcp_fast(double a) {
 }
 
 // -------------------------------------------------------------------------- per-CTA workspace
+// One Clifford on (q0, q1) (q1 = q0 for one qudit): the exponents of its generator images, generator k's at
+// a[4 k .. 4 k + 3] in the order x_q0, z_q0, x_q1, z_q1, and their phases r; s = z(g_k) . x(g_l) for k <= l, in row
+// order; inv: the images of its inverse, 4 exponents and the phase each.
+constexpr int kGates = 64;   // gates on disjoint qudits are at most kMaxN / 2
+struct GateTab {
+  uint8_t a[16], r[4], s[10], inv[20];
+  uint8_t q0, q1, ng;        // ng: generators, 2 or 4
+};
 struct Smem {
-  uint8_t lut[81 * 5];        // conjugation table of the current two-qudit Clifford
-  int img[20];                // its generator images, 4 x (x0, z0, x1, z1, r)
-  int inv[20];                // images of its inverse
-  uint8_t src[4][2 * kMaxN];  // rows read by a row product
-  int srcr[4];
   double s2[kMaxK];           // Renyi-2 entropy per class (cluster leader)
   double vn[kMaxK];           // von Neumann entropy per class (cluster leader)
   uint8_t evald[kMaxK];       // vn[k] valid
@@ -218,6 +221,12 @@ struct Smem {
       float2 whv[kWarps][32], whw[kWarps][32];   // the same per warp (warp-level estimates, m <= 32)
     };
     double2 z[kZ];              // small factorisations: the matrix, column by column
+    struct {                      // Cliffords on disjoint qudits
+      GateTab gate[kGates];
+      int ph[2 * kMaxN];          // phase each row gains
+      int first[kMaxN];           // first gate of the window on a qudit
+      int nlead;                  // gates before the first that shares a qudit with an earlier one
+    };
   };
   float redh[2][kWarps / 2];    // partial sums of the half-CTA groups
   int jmode, jm, jn;          // cluster split of a bond visit: 0 none, 2 cluster Jacobi; its matrix shape (leader)
@@ -406,180 +415,224 @@ __device__ void block_matmul(double2* Cm, const double2* A, const double2* B, in
 }
 
 // ------------------------------------------------------------------------- tableau (Sec. 2.3)
-// Images are normalised to 4 x (x0, z0, x1, z1, r); for one qudit only generators 0, 1 are used
-// and x1 = z1 = 0.
+// Gates on disjoint qudits commute and touch disjoint columns (conjugated rows) or rows (row products) of a tableau,
+// so a whole brickwork layer goes at once: a thread per (row, gate), a warp per gate's rows, four barriers.  Gate by
+// gate, each with a d^4-entry table, a layer of 48 gates on 96 qutrits took 650 kcycles, bound by the barriers
+// and by reads of a few bytes each.
 
-// lut[v] = exponents and phase of G W(v) G^dag for every local exponent vector v, where
-// W(v) = X_q0^v0 Z_q0^v1 X_q1^v2 Z_q1^v3 and the images of the generators are s.img.  The product of
-// images is accumulated with the Weyl rule  (tau^r W(a))(tau^r' W(b)) = tau^{r+r'+2 sum z(a) x(b)} W(a+b).
-__device__ void lut_build(Smem& s, int nq, int d) {
-  const int ng = 2 * nq;
-  int nent = d * d;
-  if (nq == 2) nent *= d * d;
-  for (int v = threadIdx.x; v < nent; v += blockDim.x) {
-    int dig[4] = {0, 0, 0, 0};
-    int t = v;
-    for (int k = ng - 1; k >= 0; --k) {
-      dig[k] = t % d;
-      t /= d;
-    }
-    int ax0 = 0, az0 = 0, ax1 = 0, az1 = 0, r = 0;
-    for (int k = 0; k < ng; ++k) {
-      const int* g = s.img + 5 * k;
-      for (int p = 0; p < dig[k]; ++p) {
-        r += g[4] + 2 * (az0 * g[0] + az1 * g[2]);
-        ax0 = (ax0 + g[0]) % d;
-        az0 = (az0 + g[1]) % d;
-        ax1 = (ax1 + g[2]) % d;
-        az1 = (az1 + g[3]) % d;
+// Phase (units of tau) of prod_k (tau^{r_k} W(g_k))^{v_k}, the product taken in the order of k with the Weyl rule
+// (tau^r W(a)) (tau^r' W(b)) = tau^{r + r' + 2 z(a) . x(b)} W(a + b), s as in GateTab.
+template <class R, class S>
+__device__ __forceinline__ int product_phase(const int v[4], const R& r, const S& s) {
+  int ph = 0, t = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    ph += v[k] * r[k] + v[k] * (v[k] - 1) * s[t++];
+#pragma unroll
+    for (int l = k + 1; l < 4; ++l) ph += 2 * v[k] * v[l] * s[t++];
+  }
+  return ph;
+}
+
+// The table of the Clifford with images img (gcamps_apply_clifford's layout).  The inverse's image of a generator e
+// has the exponents v with sum_k v_k g_k = e: by the symplectic form, v on X_q is Lambda(g_{Z_q}, e) and on Z_q
+// -Lambda(g_{X_q}, e); its phase undoes that product's.
+template <int D>
+__device__ void gate_table(GateTab& g, const int32_t* img, int q0, int q1) {
+  const bool two = q1 >= 0;
+  int a[4][4], r[4], s[10];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) a[k][c] = two ? img[5 * k + c] : (k < 2 && c < 2 ? img[3 * k + c] : 0);
+    r[k] = two ? img[5 * k + 4] : (k < 2 ? img[3 * k + 2] : 0);
+  }
+  int t = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int l = k; l < 4; ++l) s[t++] = (a[k][1] * a[l][0] + a[k][3] * a[l][2]) % D;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) g.a[4 * k + c] = (uint8_t)a[k][c];
+    g.r[k] = (uint8_t)r[k];
+  }
+#pragma unroll
+  for (int i = 0; i < 10; ++i) g.s[i] = (uint8_t)s[i];
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    int v[4];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {   // Lambda(u, X_p) = z_p(u), Lambda(u, Z_p) = -x_p(u)
+      const int p = h >> 1;
+      if ((h & 1) == 0) {
+        v[2 * q] = a[2 * q + 1][2 * p + 1];
+        v[2 * q + 1] = (D - a[2 * q][2 * p + 1]) % D;
+      } else {
+        v[2 * q] = (D - a[2 * q + 1][2 * p]) % D;
+        v[2 * q + 1] = a[2 * q][2 * p];
       }
     }
-    uint8_t* o = s.lut + 5 * v;
-    o[0] = (uint8_t)ax0;
-    o[1] = (uint8_t)az0;
-    o[2] = (uint8_t)ax1;
-    o[3] = (uint8_t)az1;
-    o[4] = (uint8_t)(r % (2 * d));
+    const int ph = product_phase(v, r, s) % (2 * D);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) g.inv[5 * h + k] = (uint8_t)v[k];
+    g.inv[5 * h + 4] = (uint8_t)((2 * D - ph) % (2 * D));
   }
+  g.q0 = (uint8_t)q0;
+  g.q1 = (uint8_t)(two ? q1 : q0);
+  g.ng = two ? 4 : 2;
+}
+
+// s.gate[0 .. ng) (disjoint qudits, written before the call without a barrier): every row of (cx, cr) is conjugated
+// by the gates; on (px, pr) the rows of each gate's generators (row n + q of X_q, q of Z_q) become the products of
+// old rows that its inverse images name.
+template <int D>
+__device__ void tableau_gates(Smem& s, const Ctx& C, int ng, uint8_t* cx, uint8_t* cr, uint8_t* px, uint8_t* pr) {
+  const int n = C.n, len = 2 * n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < len; i += blockDim.x) s.ph[i] = 0;
   __syncthreads();
-  // Inverse images: the unique v with G W(v) G^dag = tau^delta g_k gives G^dag g_k G = tau^{-delta} W(v).
-  for (int v = threadIdx.x; v < nent; v += blockDim.x) {
-    const uint8_t* o = s.lut + 5 * v;
-    int hit = -1, cnt = 0;
+  constexpr int kPer = (kMaxN + 31) / 32;
+  for (int t = kWarps - 1 - warp; t < ng; t += kWarps) {   // a single gate: the last warp, the first ones conjugate
+    const GateTab& g = s.gate[t];
+    const int gens = g.ng;
+    int x[4][kPer], z[4][kPer], r[4], row[4];
+#pragma unroll
     for (int k = 0; k < 4; ++k) {
-      if (o[k]) {
-        ++cnt;
-        hit = (o[k] == 1) ? k : -2;
+      const int q = (k >> 1) ? g.q1 : g.q0;
+      row[k] = (k & 1) ? q : n + q;
+      const uint8_t* R = px + row[k] * len;
+      r[k] = k < gens ? pr[row[k]] : 0;
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        const int j = lane + 32 * u;
+        const bool in = k < gens && j < n;
+        x[k][u] = in ? R[j] : 0;
+        z[k][u] = in ? R[n + j] : 0;
       }
     }
-    if (cnt == 1 && hit >= 0 && hit < ng) {
-      int dig[4] = {0, 0, 0, 0};
-      int t = v;
-      for (int k = ng - 1; k >= 0; --k) {
-        dig[k] = t % d;
-        t /= d;
-      }
-      int* w = s.inv + 5 * hit;
-      for (int k = 0; k < 4; ++k) w[k] = dig[k];
-      w[4] = (2 * d - o[4]) % (2 * d);
-    }
-  }
-  __syncthreads();
-}
-
-// Conjugate every row of a tableau by the Clifford of s.lut on sites q0 (, q1).
-__device__ void tab_apply_lut(Smem& s, uint8_t* X, uint8_t* R, int n, int d, int q0, int q1, int nq) {
-  for (int row = threadIdx.x; row < 2 * n; row += blockDim.x) {
-    uint8_t* e = X + (long long)row * 2 * n;
-    int v = e[q0] * d + e[n + q0];
-    if (nq == 2) v = (v * d + e[q1]) * d + e[n + q1];
-    const uint8_t* o = s.lut + 5 * v;
-    e[q0] = o[0];
-    e[n + q0] = o[1];
-    if (nq == 2) {
-      e[q1] = o[2];
-      e[n + q1] = o[3];
-    }
-    R[row] = (uint8_t)((R[row] + o[4]) % (2 * d));
-  }
-  __syncthreads();
-}
-
-// Replace the rows of the generators on (q0, q1) by products of the old rows: row(g_k) becomes
-// tau^{r_k} prod_g row(g)^{v_k[g]} for the images (v_k, r_k) in s.inv (generator order
-// X_q0, Z_q0, X_q1, Z_q1; row of X_q is n + q, of Z_q is q).
-__device__ void tab_rowprod(Smem& s, uint8_t* X, uint8_t* R, int n, int d, int q0, int q1, int nq) {
-  const int ng = 2 * nq;
-  const int rowlen = 2 * n;
-  for (int i = threadIdx.x; i < ng * rowlen; i += blockDim.x) {
-    const int g = i / rowlen, j = i % rowlen;
-    const int q = (g >> 1) ? q1 : q0;
-    const int row = (g & 1) ? q : n + q;
-    s.src[g][j] = X[(long long)row * rowlen + j];
-  }
-  if (threadIdx.x < ng) {
-    const int g = threadIdx.x;
-    const int q = (g >> 1) ? q1 : q0;
-    s.srcr[g] = R[(g & 1) ? q : n + q];
-  }
-  __syncthreads();
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (w < ng) {
-    constexpr int kPer = (kMaxN + 31) / 32;
-    int ax[kPer], az[kPer];
+    // z(row_k) . x(row_l), three sums of at most 4 kMaxN to a word
+    int dot[10];
+    {
+      unsigned w[4] = {0, 0, 0, 0};
+      int i = 0;
 #pragma unroll
-    for (int t = 0; t < kPer; ++t) ax[t] = az[t] = 0;
-    int r = s.inv[5 * w + 4];
-    for (int g = 0; g < ng; ++g) {
-      const int pw = s.inv[5 * w + g];
-      for (int p = 0; p < pw; ++p) {
-        int loc = 0;
+      for (int k = 0; k < 4; ++k)
 #pragma unroll
-        for (int t = 0; t < kPer; ++t) {
-          const int j = lane + 32 * t;
-          if (j < n) loc += az[t] * s.src[g][j];
+        for (int l = k; l < 4; ++l, ++i) {
+          int acc = 0;
+#pragma unroll
+          for (int u = 0; u < kPer; ++u) acc += z[k][u] * x[l][u];
+          w[i / 3] |= (unsigned)acc << (10 * (i % 3));
         }
-        r += s.srcr[g] + 2 * warp_sum_int(loc);
 #pragma unroll
-        for (int t = 0; t < kPer; ++t) {
-          const int j = lane + 32 * t;
-          if (j < n) {
-            ax[t] = (ax[t] + s.src[g][j]) % d;
-            az[t] = (az[t] + s.src[g][n + j]) % d;
-          }
+      for (int c = 0; c < 4; ++c) w[c] = __reduce_add_sync(0xffffffffu, w[c]);
+#pragma unroll
+      for (i = 0; i < 10; ++i) dot[i] = (w[i / 3] >> (10 * (i % 3))) & 1023;
+    }
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      if (h >= gens) break;
+      int v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = k < gens ? g.inv[5 * h + k] : 0;
+      uint8_t* R = px + row[h] * len;
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        const int j = lane + 32 * u;
+        if (j < n) {
+          R[j] = (uint8_t)((v[0] * x[0][u] + v[1] * x[1][u] + v[2] * x[2][u] + v[3] * x[3][u]) % D);
+          R[n + j] = (uint8_t)((v[0] * z[0][u] + v[1] * z[1][u] + v[2] * z[2][u] + v[3] * z[3][u]) % D);
         }
       }
+      if (lane == 0) pr[row[h]] = (uint8_t)((g.inv[5 * h + 4] + product_phase(v, r, dot)) % (2 * D));
     }
-    const int q = (w >> 1) ? q1 : q0;
-    const int row = (w & 1) ? q : n + q;
+  }
+  for (int idx = threadIdx.x; idx < len * ng; idx += blockDim.x) {
+    const int row = idx / ng;
+    const GateTab& g = s.gate[idx - row * ng];
+    uint8_t* e = cx + row * len;
+    int v[4];
+    v[0] = e[g.q0];
+    v[1] = e[n + g.q0];
+    v[2] = g.ng == 4 ? e[g.q1] : 0;
+    v[3] = g.ng == 4 ? e[n + g.q1] : 0;
+    if ((v[0] | v[1] | v[2] | v[3]) == 0) continue;
+    int o[4];
 #pragma unroll
-    for (int t = 0; t < kPer; ++t) {
-      const int j = lane + 32 * t;
-      if (j < n) {
-        X[(long long)row * rowlen + j] = (uint8_t)ax[t];
-        X[(long long)row * rowlen + n + j] = (uint8_t)az[t];
-      }
+    for (int c = 0; c < 4; ++c) o[c] = (v[0] * g.a[c] + v[1] * g.a[4 + c] + v[2] * g.a[8 + c] + v[3] * g.a[12 + c]) % D;
+    e[g.q0] = (uint8_t)o[0];
+    e[n + g.q0] = (uint8_t)o[1];
+    if (g.ng == 4) {
+      e[g.q1] = (uint8_t)o[2];
+      e[n + g.q1] = (uint8_t)o[3];
     }
-    if (lane == 0) R[row] = (uint8_t)(((r % (2 * d)) + 2 * d) % (2 * d));
+    const int ph = product_phase(v, g.r, g.s) % (2 * D);
+    if (ph) atomicAdd(&s.ph[row], ph);
   }
+  __syncthreads();
+  for (int i = threadIdx.x; i < len; i += blockDim.x)
+    if (s.ph[i]) cr[i] = (uint8_t)((cr[i] + s.ph[i]) % (2 * D));
   __syncthreads();
 }
 
-__device__ void load_images(Smem& s, const int32_t* img, int nq) {
-  if (threadIdx.x < 20) {
-    int v = 0;
-    const int k = threadIdx.x / 5, f = threadIdx.x % 5;
-    if (nq == 2) {
-      v = img[threadIdx.x];
-    } else if (k < 2) {
-      if (f == 0) v = img[3 * k + 0];
-      else if (f == 1) v = img[3 * k + 1];
-      else if (f == 4) v = img[3 * k + 2];
+// C <- G C (Sec. 3, top loop of Fig. 3) for count Clifford gates in order: forward rows conjugated by G, the rows of
+// the inverse tableau for G's sites replaced by products of old rows.  Each step takes the longest run of gates on
+// disjoint qudits.
+template <int D>
+__device__ void clifford_steps(Smem& s, const Ctx& C, const gcamps_op* ops, int count) {
+  const int tid = threadIdx.x;
+  for (int p = 0; p < count;) {
+    const int w = min(count - p, kGates);
+    for (int q = tid; q < C.n; q += blockDim.x) s.first[q] = kGates;
+    if (tid == 0) s.nlead = w;
+    __syncthreads();
+    int q0 = 0, q1 = -1;
+    if (tid < w) {
+      q0 = ops[p + tid].q0;
+      q1 = ops[p + tid].q1;
+      atomicMin(&s.first[q0], tid);
+      if (q1 >= 0) atomicMin(&s.first[q1], tid);
     }
-    s.img[threadIdx.x] = v;
-    s.inv[threadIdx.x] = 0;
+    __syncthreads();
+    if (tid < w && (s.first[q0] < tid || (q1 >= 0 && s.first[q1] < tid))) atomicMin(&s.nlead, tid);
+    __syncthreads();
+    const int ng = s.nlead;
+    if (tid < ng) gate_table<D>(s.gate[tid], ops[p + tid].img, q0, q1);
+    tableau_gates<D>(s, C, ng, C.fx, C.fr, C.ix, C.ir);
+    p += ng;
   }
-  __syncthreads();
 }
-
-// C <- G C (Sec. 3, top loop of Fig. 3).  Forward rows are conjugated by G; the rows of the
-// inverse tableau for G's sites become products of old rows via the images of G^{-1}.
-__device__ void apply_clifford(Smem& s, const Ctx& C, int q0, int q1, const int32_t* img) {
-  const int nq = (q1 < 0) ? 1 : 2;
-  load_images(s, img, nq);
-  lut_build(s, nq, C.d);
-  tab_apply_lut(s, C.fx, C.fr, C.n, C.d, q0, q1, nq);
-  tab_rowprod(s, C.ix, C.ir, C.n, C.d, q0, q1, nq);
-  if (threadIdx.x == 0) C.stats[S_CLIFF] += 1;
+__device__ __noinline__ void apply_cliffords(Smem& s, const Ctx& C, const gcamps_op* ops, int count) {
+  if (C.d == 2) clifford_steps<2>(s, C, ops, count);
+  else clifford_steps<3>(s, C, ops, count);
 }
 
 // C <- C Q^dag (Sec. 3): the inverse rows are conjugated by Q, the forward rows of Q's sites
 // become products of old rows via the images of Q^{-1}.
-__device__ void fold_candidate(Smem& s, const Ctx& C, int k, int q0) {
-  load_images(s, C.e->candImg + 20 * k, 2);
-  lut_build(s, 2, C.d);
-  tab_apply_lut(s, C.ix, C.ir, C.n, C.d, q0, q0 + 1, 2);
-  tab_rowprod(s, C.fx, C.fr, C.n, C.d, q0, q0 + 1, 2);
+template <int D>
+__device__ __forceinline__ void fold_step(Smem& s, const Ctx& C, const int32_t* img, int q0) {
+  if (threadIdx.x == 0) gate_table<D>(s.gate[0], img, q0, q0 + 1);
+  tableau_gates<D>(s, C, 1, C.ix, C.ir, C.fx, C.fr);
+}
+__device__ __noinline__ void fold_candidate(Smem& s, const Ctx& C, int k, int q0) {
+  const int32_t* img = C.e->candImg + 20 * k;
+  if (C.d == 2) fold_step<2>(s, C, img, q0);
+  else fold_step<3>(s, C, img, q0);
+}
+
+// One past the last of the Clifford gates that start at ops[i] (every thread of the CTA calls it).
+__device__ int clifford_end(Smem& s, const gcamps_op* ops, int i, int stop) {
+  for (;; i += kThreads) {
+    if (threadIdx.x == 0) s.flag = kThreads;
+    __syncthreads();
+    const int k = i + (int)threadIdx.x;
+    if (k >= stop || ops[k].kind != GCAMPS_OP_CLIFFORD) atomicMin(&s.flag, (int)threadIdx.x);
+    __syncthreads();
+    const int f = s.flag;
+    __syncthreads();
+    if (f < kThreads) return i + f;
+  }
 }
 
 // --------------------------------------------------------- one-sided Jacobi SVD (block level)
@@ -3775,11 +3828,15 @@ __device__ void init_tau(Smem& s, int d) {
 }
 
 // Clifford and non-Clifford steps touch only the leader's state; disentangling uses the cluster.
-__device__ void run_op(Smem& s, Smem* lead, const Ctx& C, const gcamps_op& op) {
+// ncliff: Clifford gates taken at once from a Clifford op on.
+__device__ void run_op(Smem& s, Smem* lead, const Ctx& C, const gcamps_op& op, int ncliff = 1) {
   long long tp = prof_start(C);
   switch (op.kind) {
     case GCAMPS_OP_CLIFFORD:
-      if (C.rank == 0) apply_clifford(s, C, op.q0, op.q1, op.img);
+      if (C.rank == 0) {
+        apply_cliffords(s, C, &op, ncliff);
+        if (threadIdx.x == 0) C.stats[S_CLIFF] += ncliff;
+      }
       prof_lap(C, P_CLIFF, tp);
       break;
     case GCAMPS_OP_NONCLIFFORD:
@@ -3857,7 +3914,11 @@ __device__ __forceinline__ void run_body(const Engine& e, const gcamps_op* ops, 
     e.prof[(long long)c * P_COUNT + P_SMID + rank] = 1 + (long long)sm;
   }
   if (GCAMPS_TC && e.tc_smem) tc_setup(s);
-  for (int i = first; i < stop; ++i) run_op(s, lead, C, ops[i]);
+  for (int i = first; i < stop;) {
+    const int end = max(clifford_end(s, ops, i, stop), i + 1);
+    run_op(s, lead, C, ops[i], end - i);
+    i = end;
+  }
   store_counters(s, C);
   cluster_sync();
   if (GCAMPS_TC && e.tc_smem) tc_teardown(s);
