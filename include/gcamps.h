@@ -377,8 +377,8 @@ int gcamps_estimate_theta(gcamps_t* h, int chi_l, int chi_r, const double* theta
  * counterpart of this call; it is a deployment variant of the disentangler scoring.
  *
  * It needs no handle and allocates nothing (no cudaMalloc, no cudaFree, no allocating library
- * routine).  Its working memory is one static device array of this library, 1,696,256 bytes, that
- * every GPU which loads the library holds until the process exits.  That array fixes the largest
+ * routine).  Its working memory is one static device array of this library, 19,072 bytes, that
+ * every GPU which loads the library holds until the process exits, and a CTA's shared memory, which fixes the largest
  * tensor: chi_l d <= GCAMPS_NOALLOC_MAX_SIDE and d chi_r <= GCAMPS_NOALLOC_MAX_SIDE, i.e. chi <= 27
  * for qutrits and chi <= 40 for qubits; a larger shape returns GCAMPS_ESIZE and launches nothing.
  *

@@ -276,12 +276,14 @@ struct Ctx {
   double2* scr;
   double* sing;
   int* perm;
+  const double* known;        // scores of every class taken beforehand (KnownScore; null: they are evaluated)
 };
 
 __device__ __forceinline__ double2* site_ptr(const Ctx& C, int j) { return C.mps + C.site_off[j]; }
 
 __device__ Ctx make_ctx(const Engine& e, int c, int rank = 0) {
   Ctx C;
+  C.known = nullptr;
   C.e = &e;
   C.c = c;
   C.rank = rank;
@@ -3031,6 +3033,10 @@ __device__ void gram_fp32<BlockGroup>(const BlockGroup& g, const Ctx& C, const f
 // kS2Exact: S2 in FP64 only (class 0 still gets kExact: its eigenvalues certify QR moves).
 // kPurity: S2 in FP64 only, for every listed class and in the precision form too.
 // kEstimate: the FP32 von Neumann estimate and its bound (lead->vest, lead->vbd; CTA-level sizes only).
+// Where scores of every class were taken beforehand (one CTA a class: k_score_grid), they are looked up: rows of kMaxK
+// doubles, FP64 S2, S_vN and weight rank, FP32 S2 and its lower bound, FP32 estimate and its error bound.
+enum KnownScore { kKnownS2 = 0, kKnownVn, kKnownRank, kKnownScreen, kKnownScreenLo, kKnownEst, kKnownBound, kKnownRows };
+static_assert(kKnownRows * kMaxK <= kScoreWork, "known scores fit");
 enum ScoreMode { kExact = 0, kScreen = 1, kS2Exact = 2, kEstimate = 3, kPurity = 4 };
 __device__ void score_classes(Smem& s, Smem* lead, const Ctx& C, const double2* theta, int cl, int cr,
                               const int* list, int cnt, int mode) {
@@ -3038,6 +3044,31 @@ __device__ void score_classes(Smem& s, Smem* lead, const Ctx& C, const double2* 
   const int d = C.d, dd = d * d;
   const int rows = cl * d, cols = d * cr;
   const int m = rows < cols ? rows : cols;
+  if (C.known) {
+    const bool warp_level = (long long)rows * cols <= kSmall && m * m <= kSmall;
+    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
+      const int k = list ? list[t] : t;
+      auto row = [&](KnownScore r) { return C.known[r * kMaxK + k]; };
+      if (mode == kScreen || (mode == kEstimate && warp_level)) {
+        s.s2[k] = row(kKnownScreen);
+        s.s2lo[k] = row(kKnownScreenLo);
+      }
+      if (mode == kEstimate) {
+        s.vest[k] = row(kKnownEst);
+        s.vbd[k] = row(kKnownBound);
+        s.estd[k] = 1;
+      }
+      if (mode == kExact || mode == kS2Exact) {
+        const bool want_vn = mode == kExact || k == 0;
+        s.s2[k] = row(kKnownS2);
+        s.evald[k] = 1;
+        s.vn[k] = want_vn ? row(kKnownVn) : CUDART_NAN;
+        s.rk[k] = want_vn ? (int)row(kKnownRank) : -1;
+        if (k == 0) s.rank0 = s.rk[k];
+      }
+    }
+    return;
+  }
   // exact evaluations at warp-level sizes run one per CTA when the list has no more entries than the
   // cluster has CTAs and m >= exact_cta_min_m: a CTA spreads one evaluation over its four FP64 pipes
   const bool cta_exact = mode == kExact && cnt <= C.csize && m >= e.exact_cta_min_m;
@@ -3301,7 +3332,7 @@ __device__ int select_class(Smem& s, Smem* lead, const Ctx& C, const double2* th
     if (est_kind) s.dval[3] = vn_est_bound(d, m, rows < cols ? cols : rows);
   }
   if (prune) {   // FP32 copy of theta for the screen, shared by the cluster
-    if (leader)
+    if (leader && !C.known)
       for (int i = threadIdx.x; i < rows * cols; i += blockDim.x)
         C.th32[i] = make_float2((float)theta[i].x, (float)theta[i].y);
     cluster_sync();

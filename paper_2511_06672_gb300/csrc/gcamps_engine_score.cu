@@ -1,5 +1,8 @@
-// Class scoring on a given two-site tensor (arxiv 2511.06672, Sec. 3): the handle-based kernel and the
-// variant whose working memory is a static device array of the library (no allocation).
+// Class scoring on a given two-site tensor (arxiv 2511.06672, Sec. 3): a CTA per class for tensors whose work fits
+// shared memory, the engine's cluster kernel for larger ones, and the variant whose working memory is a static
+// device array of the library (no allocation).
+
+#include <algorithm>
 
 #include "gcamps_device.cuh"
 
@@ -41,6 +44,167 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) k_estimate_theta(Engine e,
   cluster_sync();
 }
 
+// theta' = Q theta and its Gram, `width` columns of the long side at a time: x holds the short side's m entries of each
+// (short index major, padded stride, where the rows are short; long index major where the columns are).
+template <class Grp>
+__device__ void gram_chunked(const Grp& g, const double2* theta, int cl, int cr, int d, const double2* Q, double2* G,
+                             double2* x, int width) {
+  const int dd = d * d, rows = cl * d, cols = d * cr;
+  const bool wide = rows <= cols;
+  const int m = wide ? rows : cols, M = wide ? cols : rows, ntri = m * (m + 1) / 2;
+  const int ld = wide ? (width | 1) : m;
+  for (int c0 = 0; c0 < M; c0 += width) {
+    const int w = min(width, M - c0);
+    for (int idx = g.tid; idx < m * w; idx += g.n) {
+      const int i = wide ? idx / w : idx % m, c = wide ? idx % w : idx / m;
+      const int rr = wide ? i : c0 + c, col = wide ? c0 + c : i;
+      const int a = rr / d, sd = rr % d, t = col / cr, b = col % cr;
+      const double2* q = Q + (sd * d + t) * dd;
+      const double2* th = theta + (long long)a * dd * cr + b;
+      double2 acc = cz();
+      for (int u = 0; u < dd; ++u) acc = cfma(q[u], th[(long long)u * cr], acc);
+      x[wide ? i * ld + c : c * ld + i] = acc;
+    }
+    g.sync();
+    for (int idx = g.tid; idx < ntri; idx += g.n) {
+      int i, j;
+      tri_index(idx, i, j);
+      double2 acc = c0 ? G[i * m + j] : cz();
+      if (wide)
+        for (int c = 0; c < w; ++c) acc = cfmac(x[j * ld + c], x[i * ld + c], acc);   // sum_c x_i conj(x_j)
+      else
+        for (int c = 0; c < w; ++c) acc = cfmac(x[c * ld + i], x[c * ld + j], acc);
+      G[i * m + j] = acc;
+      if (c0 + width >= M && i != j) G[j * m + i] = cconj(acc);
+    }
+    g.sync();
+  }
+}
+
+// Every class of one theta at once: CTA k < K takes the exact FP64 scores of class k, CTA K + k its FP32 screen and
+// estimate, into rows of kMaxK doubles (KnownScore).  The classes are independent, and 90 CTAs on 152 SMs take the
+// time of one: at m = 81 2 ms instead of 38 ms for the classes in turn on a cluster of 4.  theta', the Gram and the
+// reduction's scratch live in dynamic shared memory (kGridMax entries of theta).  Below kGridWarpM rows a CTA is one
+// warp (the steps of a reduction of so few rows fit one).
+constexpr int kGridMax = 81 * 81, kGridWarpM = 10, kGridWidth = 32;
+template <class Grp>
+__device__ __forceinline__ void score_grid_body(Smem& s, const Grp& g, const Engine& e, const double2* th, int cl,
+                                                int cr, double* out) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  Ctx C = {};
+  C.e = &e;
+  C.d = e.d;
+  C.K = e.K;
+  C.rank = 1;   // not a leader: no counters
+  const int d = e.d, dd = d * d, rows = cl * d, cols = d * cr;
+  const int m = min(rows, cols), M = max(rows, cols);
+  const int k = blockIdx.x % e.K;
+  constexpr bool kWarpLevel = Grp::kSize == 32;
+  if (blockIdx.x < e.K) {
+    double2* G = reinterpret_cast<double2*>(dyn);
+    double* dg = reinterpret_cast<double*>(G + m * m);
+    double* od = dg + m;
+    gram_chunked(g, th, cl, cr, d, e.candU + (long long)k * dd * dd, G, G + m * m + m, min(M, kGridWidth));
+    double tr = 0, fro = 0;
+    for (int idx = g.tid; idx < m * m; idx += g.n) {
+      const double2 v = G[idx];
+      if (idx / m == idx % m) tr += v.x;
+      fro += cabs2(v);
+    }
+    tr = g.sum(tr);
+    fro = g.sum(fro);
+    const Score sc = score_spectrum(g, C, G, m, tr, fro, true, dg, od, kWarpLevel ? s.wtri[0] : s.btri,
+                                    kWarpLevel ? s.wtri32[0] : s.btri32, kWarpLevel ? 32 : kBTri);
+    if (g.tid == 0) {
+      out[kKnownS2 * kMaxK + k] = sc.s2;
+      out[kKnownVn * kMaxK + k] = sc.vn;
+      out[kKnownRank * kMaxK + k] = sc.rank;
+    }
+  } else {
+    float2* th32 = reinterpret_cast<float2*>(dyn);
+    for (int i = g.tid; i < rows * cols; i += g.n) th32[i] = make_float2((float)th[i].x, (float)th[i].y);
+    g.sync();
+    float est = 0.f, v = 0.f, lo = 0.f;
+    const bool ok = vn_est32(g, C, th32, cl, cr, e.candU32 + (long long)k * dd * dd, th32 + rows * cols,
+                             kWarpLevel ? s.whv[0] : s.hv, kWarpLevel ? s.whw[0] : s.hw, kWarpLevel ? 32 : kBTri,
+                             kWarpLevel ? s.wtri32[0] : s.btri32, kWarpLevel ? 32 : kBTri, &est, &v, &lo);
+    if (g.tid == 0) {
+      out[kKnownScreen * kMaxK + k] = v;
+      out[kKnownScreenLo * kMaxK + k] = lo;
+      out[kKnownEst * kMaxK + k] = est;
+      out[kKnownBound * kMaxK + k] = ok ? vn_est_bound(d, m, M) : 1e300;
+    }
+  }
+}
+struct GridWarp : WarpGroup {
+  static constexpr int kSize = 32;
+};
+struct GridBlock : BlockGroup {
+  static constexpr int kSize = kThreads;
+};
+__global__ void __launch_bounds__(32) k_score_grid_warp(Engine e, const double2* th, int cl, int cr, double* out) {
+  __shared__ Smem s;
+  GridWarp g;
+  g.tid = (int)threadIdx.x;
+  score_grid_body(s, g, e, th, cl, cr, out);
+}
+__global__ void __launch_bounds__(kThreads, 1) k_score_grid(Engine e, const double2* th, int cl, int cr, double* out) {
+  __shared__ Smem s;
+  GridBlock g;
+  g.s = &s;
+  g.tid = (int)threadIdx.x;
+  g.n = (int)blockDim.x;
+  score_grid_body(s, g, e, th, cl, cr, out);
+}
+
+// The disentangler's choice from the scores of k_score_grid, through select_class (e.csize as its cluster size); the
+// scores go to the caller's arrays.  choice: class, exact evaluations that the bounds leave, and (status) the device
+// status.
+__global__ void __launch_bounds__(kThreads) k_score_choice(Engine e, const double2* th, int cl, int cr,
+                                                           const double* known, double* out_s2, double* out_vn,
+                                                           int* out_choice, bool status) {
+  __shared__ Smem s;
+  Ctx C = {};
+  C.e = &e;
+  C.csize = e.csize;
+  C.d = e.d;
+  C.K = e.K;
+  C.known = known;
+  for (int k = threadIdx.x; k < C.K; k += blockDim.x) {
+    out_s2[k] = known[kKnownS2 * kMaxK + k];
+    out_vn[k] = known[kKnownVn * kMaxK + k];
+  }
+  score_classes(s, &s, C, th, cl, cr, nullptr, C.K, kExact);
+  __syncthreads();
+  int nev = 0;
+  const int kb = select_class(s, &s, C, th, cl, cr, &nev, false);
+  if (threadIdx.x == 0) {
+    out_choice[0] = kb;
+    out_choice[1] = nev;
+    if (status) out_choice[2] = 0;   // no iteration of the scoring can fail
+  }
+}
+
+// k_score_grid and k_score_choice for a theta of at most kGridMax entries; known: kKnownRows kMaxK doubles.
+cudaError_t launch_grid(const Engine& e, const double2* th, int cl, int cr, double* known, double* s2, double* vn,
+                        int* choice, bool status, cudaStream_t st) {
+  const int rows = cl * e.d, cols = e.d * cr, m = std::min(rows, cols), M = std::max(rows, cols);
+  const size_t exact = (size_t)(m * m + m + m * (std::min(M, kGridWidth) | 1)) * sizeof(double2);
+  const size_t est = (size_t)(2 * rows * cols + m * m + 3 * m) * sizeof(float2);
+  const size_t bytes = std::max(exact, est);
+  const bool warp = m < kGridWarpM;
+  auto kern = warp ? k_score_grid_warp : k_score_grid;
+  if (bytes > 16384) {   // with the static part it may exceed the 48 KB a kernel gets unasked
+    const cudaError_t a = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (a != cudaSuccess) return a;
+  }
+  kern<<<2 * e.K, warp ? 32 : kThreads, bytes, st>>>(e, th, cl, cr, known);
+  cudaError_t ce = cudaGetLastError();
+  if (ce != cudaSuccess) return ce;
+  k_score_choice<<<1, kThreads, 0, st>>>(e, th, cl, cr, known, s2, vn, choice, status);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_estimate_theta(const Engine& e, const double2* th, int cl, int cr, double* est, double* bd,
@@ -49,29 +213,23 @@ cudaError_t launch_estimate_theta(const Engine& e, const double2* th, int cl, in
 }
 
 cudaError_t launch_score_theta(const Engine& e, const double2* th, int cl, int cr, double* s2, double* vn,
-                               int* choice, cudaStream_t st) {
+                               int* choice, double* known, cudaStream_t st) {
   if (e.precision) return launch_score_theta_tc(e, th, cl, cr, s2, vn, choice, st);
+  if ((long long)cl * e.d * e.d * cr <= kGridMax) return launch_grid(e, th, cl, cr, known, s2, vn, choice, false, st);
   return launch_cluster(k_score_theta, e, st, e, th, cl, cr, s2, vn, choice);
 }
 
 // ------------------------------------------------------ class scores without device allocation
-// gcamps_score_theta_noalloc runs the scoring and the class choice of k_score_theta with all of its
-// scratch in the static array below instead of a handle's allocation.  Per CTA: kWarps warp-level
-// buffers of kSmallStride entries and one CTA-level buffer (theta' of up to kStaticSide^2 entries,
-// its Gram, eigenvalue arrays); then the last-visit score record, the status words and the FP32 copy
-// of theta used by the screen.
-constexpr long long kStaticTcap = (long long)kStaticSide * kStaticSide;
-constexpr long long kStaticCtaRaw = (long long)kWarps * kSmallStride + 2 * kStaticTcap + kStaticSide + 64;
-constexpr long long kStaticCta = (kStaticCtaRaw + 15) / 16 * 16;                  // 256-byte multiples
-constexpr long long kStaticScores = ((3LL * kMaxK + 2 + 2LL * kSmall + 1) / 2 + 15) / 16 * 16;
-constexpr long long kStaticMeta = 16;                                             // >= M_COUNT ints
-constexpr long long kStaticTh32 = ((kStaticTcap + 1) / 2 + 15) / 16 * 16;          // float2 pairs
-constexpr long long kStaticWords = kStaticCluster * kStaticCta + kStaticScores + kStaticMeta + kStaticTh32;
-static_assert(2 * kStaticMeta >= M_COUNT, "status words");
-static_assert(kStaticWords * 16 == 1696256, "scratch size stated in gcamps.h");
-// 1,696,256 bytes, held by every device that loads the library.  Calls reuse it and it keeps the
-// last call's contents; only the status words must start at zero, and each call clears them itself.
-static __device__ __align__(256) double2 g_static_scratch[kStaticWords];
+// gcamps_score_theta_noalloc: the scores of every class and the choice's record in the static array below (the rest
+// of the work is in shared memory).
+constexpr long long kStaticScores = (3LL * kMaxK + 2 + 2LL * kSmall + 15) / 16 * 16;
+constexpr long long kStaticKnown = ((long long)kKnownRows * kMaxK + 15) / 16 * 16;
+constexpr long long kStaticWords = kStaticScores + kStaticKnown;
+static_assert(kStaticWords * 8 == 19072, "scratch size stated in gcamps.h");
+static_assert(kStaticSide * kStaticSide <= kGridMax, "every accepted tensor takes the grid");
+// Held by every device that loads the library.  Calls reuse it and it keeps the last call's contents, which no
+// later call reads.
+static __device__ __align__(256) double g_static_scratch[kStaticWords];
 // Class unitaries for d = 2 then d = 3 ([K][d^4]) and their images ([K][20]), set once per device.
 static __device__ __align__(256) double2 g_static_candU[kStaticK2 * 16 + kStaticK3 * 81];
 static __device__ __align__(256) float2 g_static_candU32[kStaticK2 * 16 + kStaticK3 * 81];
@@ -80,50 +238,12 @@ static __device__ __align__(256) int32_t g_static_candImg[(kStaticK2 + kStaticK3
 // Device addresses of the arrays above, per device (host code only sees host-side stand-ins under
 // their names).
 struct StaticPtrs {
-  double2* scratch;
+  double* scratch;
   double2* candU;
   float2* candU32;
   int32_t* candImg;
 };
 static StaticPtrs g_static_ptrs[kStaticMaxDevices];
-
-// The same steps as k_score_theta for one theta; the cluster is the only one of the launch.
-__global__ void __launch_bounds__(kThreads, kMinCtas) k_score_theta_static(Engine e, const double2* th, int cl, int cr,
-                                                                 double* out_s2, double* out_vn,
-                                                                 int32_t* out_choice) {
-  __shared__ Smem s;
-  const int rank = blockIdx.x % e.csize;
-  Ctx C = {};
-  C.e = &e;
-  C.c = 0;
-  C.rank = rank;
-  C.csize = e.csize;
-  C.d = e.d;
-  C.K = e.K;
-  C.cta = e.cscr + (long long)rank * e.cl.total;
-  C.meta = e.meta;
-  C.th32 = reinterpret_cast<float2*>(e.cscr + kStaticCluster * kStaticCta + kStaticScores + kStaticMeta);
-  Smem* lead = cg::this_cluster().map_shared_rank(&s, 0);
-  init_tau(s, e.d);
-  if (rank == 0 && threadIdx.x < M_COUNT) C.meta[threadIdx.x] = 0;   // status of this call only
-  cluster_sync();
-  score_classes(s, lead, C, th, cl, cr, nullptr, C.K, kExact);
-  cluster_sync();
-  if (rank == 0)
-    for (int k = threadIdx.x; k < C.K; k += blockDim.x) {
-      out_s2[k] = s.s2[k];
-      out_vn[k] = s.vn[k];
-    }
-  cluster_sync();
-  int nev = 0;
-  const int kb = select_class(s, lead, C, th, cl, cr, &nev, false);
-  cluster_sync();
-  if (rank == 0 && threadIdx.x == 0) {
-    out_choice[0] = kb;
-    out_choice[1] = nev;
-    out_choice[2] = C.meta[M_STATUS];
-  }
-}
 
 cudaError_t static_setup(int device, const double* u2, const int32_t* img2, const double* u3,
                          const int32_t* img3) {
@@ -160,19 +280,11 @@ cudaError_t launch_score_theta_static(int device, int d, double tie_tol, const d
   e.batch = 1;
   e.csize = kStaticCluster;
   e.tie_tol = tie_tol;
-  e.tcap = kStaticTcap;
-  e.wcap = kStaticTcap;
-  e.scap = kStaticTcap;
-  e.cscr = p.scratch;
-  e.cl.warp = 0;
-  e.cl.block = (long long)kWarps * kSmallStride;
-  e.cl.total = kStaticCta;
-  e.lastsc = reinterpret_cast<double*>(p.scratch + kStaticCluster * kStaticCta);
-  e.meta = reinterpret_cast<int*>(p.scratch + kStaticCluster * kStaticCta + kStaticScores);
+  e.lastsc = p.scratch;
   e.candU = p.candU + (d == 2 ? 0 : kStaticK2 * 16);
   e.candU32 = p.candU32 + (d == 2 ? 0 : kStaticK2 * 16);
   e.candImg = p.candImg + (d == 2 ? 0 : kStaticK2 * 20);
-  return launch_cluster(k_score_theta_static, e, st, e, th, cl, cr, s2, vn, choice);
+  return launch_grid(e, th, cl, cr, p.scratch + kStaticScores, s2, vn, choice, true, st);
 }
 
 

@@ -362,6 +362,7 @@ struct gcamps {
   int8_t* xz_dev = nullptr;
   double2* out_dev = nullptr;
   double* schmidt_dev = nullptr;
+  double* score_dev = nullptr;         // gcamps_score_theta: outputs and scores (allocated by its first call)
   int* cnt_dev = nullptr;
   int* replay_dev = nullptr;           // [batch][kDecCap][2] recorded decisions to replay
   int* replay_n_dev = nullptr;         // [batch] their counts (0: choose)
@@ -762,6 +763,7 @@ void gcamps_destroy(gcamps_t* h) {
   if (h->ops_dev) cudaFree(h->ops_dev);
   if (h->begin_dev) cudaFree(h->begin_dev);
   if (h->schmidt_dev) cudaFree(h->schmidt_dev);
+  if (h->score_dev) cudaFree(h->score_dev);
   if (h->replay_dev) cudaFree(h->replay_dev);
   if (h->replay_n_dev) cudaFree(h->replay_n_dev);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -1276,20 +1278,23 @@ int gcamps_score_theta(gcamps_t* h, int chi_l, int chi_r, const double* theta, d
   if (!theta || !s2 || !vn || chi_l < 1 || chi_r < 1 || chi_l > h->e.maxdim / d || chi_r > h->e.maxdim / d)
     return fail(h, GCAMPS_EINVAL, "bad theta shape or null pointer");
   const size_t nel = (size_t)chi_l * d * d * chi_r;
-  double2* th = nullptr;
-  double* out = nullptr;
-  cudaError_t ce = cudaMalloc(&th, nel * sizeof(double2));
-  if (ce == cudaSuccess) ce = cudaMalloc(&out, (2 * gcx::kMaxK + 2) * sizeof(double));
-  if (ce == cudaSuccess) ce = cudaMemcpyAsync(th, theta, nel * sizeof(double2), cudaMemcpyHostToDevice, h->stream);
+  // theta in the Jacobi scratch of circuit 0 (wcap >= maxdim^2 entries, idle between calls); the outputs and scores
+  // in a buffer that the handle keeps
+  double2* th = h->e.scr + h->e.sl.w;
+  constexpr int kOut = 2 * gcx::kMaxK + 2;
+  if (!h->score_dev && cudaMalloc(&h->score_dev, (kOut + gcx::kScoreWork) * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(h, GCAMPS_ENOMEM, "score buffer");
+  }
+  double* out = h->score_dev;
+  cudaError_t ce = cudaMemcpyAsync(th, theta, nel * sizeof(double2), cudaMemcpyHostToDevice, h->stream);
   int* ch_dev = reinterpret_cast<int*>(out + 2 * gcx::kMaxK);
   if (ce == cudaSuccess)
-    ce = gcx::launch_score_theta(h->e, th, chi_l, chi_r, out, out + gcx::kMaxK, ch_dev, h->stream);
-  std::vector<double> host(2 * gcx::kMaxK + 2);
+    ce = gcx::launch_score_theta(h->e, th, chi_l, chi_r, out, out + gcx::kMaxK, ch_dev, out + kOut, h->stream);
+  std::vector<double> host(kOut);
   if (ce == cudaSuccess)
     ce = cudaMemcpyAsync(host.data(), out, host.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(h->stream);
-  if (th) cudaFree(th);
-  if (out) cudaFree(out);
   if (ce != cudaSuccess) return cuda_fail(h, ce, "score_theta");
   for (int k = 0; k < h->e.K; ++k) {
     s2[k] = host[k];

@@ -134,8 +134,10 @@ cudaError_t launch_expect(const Engine& e, int circuit, const int8_t* xz_dev, do
                           cudaStream_t st);
 cudaError_t launch_statevector(const Engine& e, int circuit, double2* out_dev, long long dim,
                                const int32_t* ys_dev, long long nys, void* work, cudaStream_t st);
+// known: kScoreWork doubles of device scratch
+constexpr int kScoreWork = 7 * kMaxK;
 cudaError_t launch_score_theta(const Engine& e, const double2* th, int cl, int cr, double* s2, double* vn,
-                               int* choice, cudaStream_t st);
+                               int* choice, double* known, cudaStream_t st);
 // The precision form's variants of the cluster kernels (compiled with the tensor-core Gram).
 cudaError_t launch_run_tc(const Engine& e, const gcamps_op* ops_dev, const int32_t* begin_dev, cudaStream_t st);
 cudaError_t launch_run_all_tc(const Engine& e, const gcamps_op* ops_dev, int nops, cudaStream_t st);
@@ -154,7 +156,7 @@ cudaError_t launch_adjoint(const Engine& e, int cf, int cb, const int8_t* xz_dev
 
 // gcamps_score_theta_noalloc: class scores with every scratch word in static device memory of this
 // library (no allocation).  theta is at most kStaticSide x kStaticSide (rows chi_l d, columns
-// d chi_r); kStaticCluster CTAs score it.
+// d chi_r); its pruning counts are those of a cluster of kStaticCluster CTAs.
 constexpr int kStaticSide = 81;
 static_assert(kStaticSide == GCAMPS_NOALLOC_MAX_SIDE, "limit stated in gcamps.h");
 constexpr int kStaticCluster = 4;
