@@ -3901,34 +3901,105 @@ __device__ void run_op(Smem& s, Smem* lead, const Ctx& C, const gcamps_op& op, i
 
 // P' = C^dag W C for W = (x)_j X_j^{x_j} Z_j^{z_j} (xz = x | z): the inverse-tableau rows multiplied in
 // the order of W with the Weyl product rule; exponents into acc_x, acc_z and the phase (units of tau)
-// into *acc_r, all in shared memory.
+// into *acc_r, all in shared memory.  A thread per column: the phase is a sum over columns of (z so far) x (row's x),
+// so the columns need each other only in its total (the rows one by one, each with a CTA-wide sum, took 100 kcycles
+// at n = 32).
 __device__ void conj_weyl(Smem& s, const Ctx& C, const int8_t* xz, int* acc_x, int* acc_z, int* acc_r) {
   const int n = C.n, d = C.d;
-  for (int j = threadIdx.x; j < n; j += blockDim.x) acc_x[j] = acc_z[j] = 0;
-  if (threadIdx.x == 0) *acc_r = 0;
+  if (threadIdx.x == 0) s.ival[2] = 0;
   __syncthreads();
-  for (int q = 0; q < n; ++q) {
-    for (int kind = 0; kind < 2; ++kind) {
-      const int pw = kind == 0 ? xz[q] : xz[n + q];
-      const int rowi = kind == 0 ? n + q : q;
-      const uint8_t* R = C.ix + (long long)rowi * 2 * n;
-      for (int p = 0; p < pw; ++p) {
-        double loc = 0;
-        for (int j = threadIdx.x; j < n; j += blockDim.x) loc += acc_z[j] * R[j];
-        const int tot = (int)llround(block_sum(loc, s));
-        __syncthreads();
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-          acc_x[j] = (acc_x[j] + R[j]) % d;
-          acc_z[j] = (acc_z[j] + R[n + j]) % d;
-        }
-        if (threadIdx.x == 0) *acc_r = (*acc_r + C.ir[rowi] + 2 * tot) % (2 * d);
-        __syncthreads();
-      }
+  int ph = 0;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    int ax = 0, az = 0, cross = 0;
+#pragma unroll 4
+    for (int i = 0; i < 2 * n; ++i) {   // X_q's row n + q, then Z_q's row q
+      const int q = i >> 1, v = (i & 1) ? xz[n + q] : xz[q];
+      const uint8_t* R = C.ix + (long long)((i & 1) ? q : n + q) * 2 * n;
+      const int x = R[j], z = R[n + j];
+      cross += x * (v * az + (v * (v - 1) / 2) * z);
+      ax += v * x;
+      az += v * z;
     }
+    acc_x[j] = ax % d;
+    acc_z[j] = az % d;
+    ph += 2 * cross;
+  }
+  for (int i = threadIdx.x; i < 2 * n; i += blockDim.x) ph += (i < n ? xz[n + i] : xz[i - n]) * C.ir[i];
+  ph = warp_sum_int(ph);
+  if ((threadIdx.x & 31) == 0 && ph) atomicAdd(&s.ival[2], ph);
+  __syncthreads();
+  if (threadIdx.x == 0) *acc_r = s.ival[2] % (2 * d);
+  __syncthreads();
+}
+
+// store(o, sum_{k < K} term(o)(k)) for o < count on the CTA: P lanes share a sum, P chosen for the busiest FP64 pipe
+// (passes x warps a pipe x (4 ceil(K / P) multiply-adds + 2 log2 P adds)).
+template <class Term, class Store>
+__device__ __forceinline__ void split_sums(int count, int K, Term term, Store store) {
+  int P = 1, best = 1 << 30;
+  for (int q = 1, lg = 0; q <= 32 && (q == 1 || q <= K); q *= 2, ++lg) {
+    const int outs = kThreads / q, passes = (count + outs - 1) / outs;
+    const int warps = min(kWarps, (min(count, outs) * q + 31) / 32);
+    const int cost = passes * ((warps + 3) / 4) * (4 * ((K + q - 1) / q) + 2 * lg);
+    if (cost < best) {
+      best = cost;
+      P = q;
+    }
+  }
+  const int outs = kThreads / P, c = threadIdx.x & (P - 1);
+  for (int base = 0; base < count; base += outs) {
+    const int o = base + (int)threadIdx.x / P;
+    double2 acc = cz();
+    if (o < count) {
+      const auto t = term(o);
+      for (int k = c; k < K; k += P) acc = t(k, acc);
+    }
+    for (int h = P >> 1; h > 0; h >>= 1) {
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, h);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, h);
+    }
+    if (o < count && c == 0) store(o, acc);
   }
 }
 
-
+// One site of <A| X^x Z^z |M>: E[a, a'] (bl x ml) becomes E'[b, b'] (br x mr), in place, through
+// T[a, s, b'] = sum_{a'} E[a, a'] omega^{z (s - x)} M[a', s - x, b'],  E'[b, b'] = sum_{a, s} conj(A[a, s, b]) T[a, s, b'].
+// next: the following site's tensors, fetched towards the SM meanwhile (null: none).
+__device__ void transfer_site(Smem& s, double2* E, double2* T, const double2* A, int bl, int br, const double2* M, int ml,
+                              int mr, int d, int x, int z, const double2* next, int next_count) {
+  if (next && (int)threadIdx.x * 8 < next_count)
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(next + threadIdx.x * 8));
+  split_sums(bl * d * mr, ml,
+             [&](int o) {
+               const int bp = o % mr, sd = (o / mr) % d, a = o / (mr * d);
+               const int sp = sd >= x ? sd - x : sd - x + d;
+               const double2* e = E + (long long)a * ml;
+               const double2* m = M + (long long)sp * mr + bp;
+               return [=](int k, double2 acc) { return cfma(e[k], m[(long long)k * d * mr], acc); };
+             },
+             [&](int o, double2 acc) {
+               const int sd = (o / mr) % d, sp = sd >= x ? sd - x : sd - x + d;
+               const int ph = (2 * z * sp) % (2 * d);
+               T[o] = ph ? cmul(s.tau[ph], acc) : acc;
+             });
+  __syncthreads();
+  split_sums(br * mr, bl * d,
+             [&](int o) {
+               const double2* a = A + o / mr;
+               const double2* t = T + o % mr;
+               return [=](int k, double2 acc) { return cfmac(a[(long long)k * br], t[(long long)k * mr], acc); };
+             },
+             [&](int o, double2 acc) { E[o] = acc; });
+  __syncthreads();
+}
+// Shared memory for E and T where every bond of both states allows it: bra bond dimensions ba, ket ones bk.
+constexpr int kTransferE = 200;   // E's part of s.z
+__device__ __forceinline__ bool transfer_fits(const int* ba, const int* bk, int n, int d) {
+  bool ok = true;
+  for (int j = threadIdx.x; j < n; j += blockDim.x)
+    ok = ok && ba[j + 1] * bk[j + 1] <= kTransferE && ba[j] * d * bk[j + 1] <= kZ - kTransferE;
+  return __syncthreads_and(ok);
+}
 
 // ------------------------------------------------------------ bodies of the cluster kernels
 // Each is the whole kernel: the FP64 translation units and the precision form's (GCAMPS_TC = 1) wrap them

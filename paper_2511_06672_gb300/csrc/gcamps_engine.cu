@@ -52,37 +52,17 @@ __global__ void __launch_bounds__(kThreads) k_expect(Engine e, int c, const int8
   const int n = C.n, d = e.d;
   conj_weyl(s, C, xz, acc_x, acc_z, &acc_r);
   // transfer matrices: E (chi x chi) starts as [[1]]
-  double2* E = C.scr + e.sl.b;
-  double2* T = C.scr + e.sl.tmp;
-  double2* E2 = C.scr + e.sl.u;
+  const bool fits = transfer_fits(C.dims, C.dims, n, d);
+  double2* E = fits ? s.z : C.scr + e.sl.b;
+  double2* T = fits ? s.z + kTransferE : C.scr + e.sl.tmp;
   if (threadIdx.x == 0) E[0] = make_double2(1.0, 0.0);
   __syncthreads();
   for (int j = 0; j < n; ++j) {
     const int cl = C.dims[j], cr = C.dims[j + 1];
     const double2* A = site_ptr(C, j);
-    const int a_j = acc_x[j], b_j = acc_z[j];
-    // T[a, s, b'] = sum_{a'} E[a, a'] (X^a Z^b A)[a', s, b'],  (X^a Z^b A)[a', s, b'] = omega^{b (s-a)} A[a', s-a, b']
-    for (long long idx = threadIdx.x; idx < (long long)cl * d * cr; idx += blockDim.x) {
-      const int bp = (int)(idx % cr), sd = (int)((idx / cr) % d), a = (int)(idx / ((long long)cr * d));
-      const int sp = (sd - a_j + d) % d;
-      const double2 ph = s.tau[(2 * b_j * sp) % (2 * d)];
-      double2 acc = cz();
-      for (int ap = 0; ap < cl; ++ap) acc = cfma(E[(long long)a * cl + ap], A[((long long)ap * d + sp) * cr + bp], acc);
-      T[idx] = cmul(ph, acc);
-    }
-    __syncthreads();
-    // E'[b, b'] = sum_{a, s} conj(A[a, s, b]) T[a, s, b']
-    for (long long idx = threadIdx.x; idx < (long long)cr * cr; idx += blockDim.x) {
-      const int b = (int)(idx / cr), bp = (int)(idx % cr);
-      double2 acc = cz();
-      for (int a = 0; a < cl; ++a)
-        for (int sd = 0; sd < d; ++sd)
-          acc = cfmac(A[((long long)a * d + sd) * cr + b], T[((long long)a * d + sd) * cr + bp], acc);
-      E2[idx] = acc;
-    }
-    __syncthreads();
-    block_copy(E, E2, (long long)cr * cr);
-    __syncthreads();
+    const bool more = j + 1 < n;
+    transfer_site(s, E, T, A, cl, cr, A, cl, cr, d, acc_x[j], acc_z[j], more ? site_ptr(C, j + 1) : nullptr,
+                  more ? cr * d * C.dims[j + 2] : 0);
   }
   if (threadIdx.x == 0) out[0] = cmul(s.tau[acc_r], E[0]);
 }
@@ -255,31 +235,17 @@ __global__ void k_apply_clifford_dense(Engine e, int c, long long dim, const dou
 // E[a1][a2] from the left, T[a1][s][b2] = sum_a2 E[a1][a2] B[a2][s][b2], then
 // E'[b1][b2] = sum_{a1, s} conj(A[a1][s][b1]) T[a1][s][b2]; FP64, one CTA, scratch of circuit c1.
 __global__ void __launch_bounds__(kThreads) k_overlap(Engine e1, int c1, Engine e2, int c2, double2* out) {
+  __shared__ Smem s;
   const Ctx A = make_ctx(e1, c1), B = make_ctx(e2, c2);
   const int n = A.n, d = e1.d;
-  double2* E = A.scr + e1.sl.b;
-  double2* T = A.scr + e1.sl.tmp;
+  const bool fits = transfer_fits(A.dims, B.dims, n, d);
+  double2* E = fits ? s.z : A.scr + e1.sl.b;
+  double2* T = fits ? s.z + kTransferE : A.scr + e1.sl.tmp;
   if (threadIdx.x == 0) E[0] = make_double2(1.0, 0.0);
   __syncthreads();
-  for (int j = 0; j < n; ++j) {
-    const int la = A.dims[j], ra = A.dims[j + 1], lb = B.dims[j], rb = B.dims[j + 1];
-    const double2* Aj = site_ptr(A, j);
-    const double2* Bj = site_ptr(B, j);
-    for (long long idx = threadIdx.x; idx < (long long)la * d * rb; idx += blockDim.x) {
-      const int a1 = (int)(idx / (d * rb)), sb = (int)(idx % (d * rb));
-      double2 acc = cz();
-      for (int a2 = 0; a2 < lb; ++a2) acc = cfma(E[(long long)a1 * lb + a2], Bj[(long long)a2 * d * rb + sb], acc);
-      T[idx] = acc;
-    }
-    __syncthreads();
-    for (long long idx = threadIdx.x; idx < (long long)ra * rb; idx += blockDim.x) {
-      const int b1 = (int)(idx / rb), b2 = (int)(idx % rb);
-      double2 acc = cz();
-      for (int as = 0; as < la * d; ++as) acc = cfmac(Aj[(long long)as * ra + b1], T[(long long)as * rb + b2], acc);
-      E[idx] = acc;
-    }
-    __syncthreads();
-  }
+  for (int j = 0; j < n; ++j)
+    transfer_site(s, E, T, site_ptr(A, j), A.dims[j], A.dims[j + 1], site_ptr(B, j), B.dims[j], B.dims[j + 1], d, 0, 0,
+                  nullptr, 0);
   if (threadIdx.x == 0) out[0] = E[0];
 }
 

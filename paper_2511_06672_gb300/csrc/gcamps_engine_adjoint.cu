@@ -13,38 +13,14 @@ __device__ double2 overlap_weyl(Smem& s, const Ctx& CB, const double2* mbase, co
                                 const long long* moff, const uint8_t* row, int mp) {
   const Engine& e = *CB.e;
   const int n = CB.n, d = CB.d;
-  double2* E = CB.scr + e.sl.b;
-  double2* T = CB.scr + e.sl.tmp;
-  double2* E2 = CB.scr + e.sl.u;
+  const bool fits = transfer_fits(CB.dims, mdims, n, d);
+  double2* E = fits ? s.z : CB.scr + e.sl.b;
+  double2* T = fits ? s.z + kTransferE : CB.scr + e.sl.tmp;
   if (threadIdx.x == 0) E[0] = make_double2(1.0, 0.0);
   __syncthreads();
-  for (int j = 0; j < n; ++j) {
-    const int bl = CB.dims[j], br = CB.dims[j + 1], ml = mdims[j], mr = mdims[j + 1];
-    const double2* A = site_ptr(CB, j);
-    const double2* M = mbase + moff[j];
-    const int ax = (mp * row[j]) % d, bz = (mp * row[n + j]) % d;
-    // T[a, s, b'] = sum_{a'} E[a, a'] omega^{bz (s - ax)} M[a', s - ax, b']
-    for (long long idx = threadIdx.x; idx < (long long)bl * d * mr; idx += blockDim.x) {
-      const int bp = (int)(idx % mr), sd = (int)((idx / mr) % d), a = (int)(idx / ((long long)mr * d));
-      const int sp = (sd - ax + d) % d;
-      double2 acc = cz();
-      for (int ap = 0; ap < ml; ++ap) acc = cfma(E[(long long)a * ml + ap], M[((long long)ap * d + sp) * mr + bp], acc);
-      T[idx] = cmul(s.tau[(2 * bz * sp) % (2 * d)], acc);
-    }
-    __syncthreads();
-    // E'[b, b'] = sum_{a, s} conj(A[a, s, b]) T[a, s, b']
-    for (long long idx = threadIdx.x; idx < (long long)br * mr; idx += blockDim.x) {
-      const int b = (int)(idx / mr), bp = (int)(idx % mr);
-      double2 acc = cz();
-      for (int a = 0; a < bl; ++a)
-        for (int sd = 0; sd < d; ++sd)
-          acc = cfmac(A[((long long)a * d + sd) * br + b], T[((long long)a * d + sd) * mr + bp], acc);
-      E2[idx] = acc;
-    }
-    __syncthreads();
-    block_copy(E, E2, (long long)br * mr);
-    __syncthreads();
-  }
+  for (int j = 0; j < n; ++j)
+    transfer_site(s, E, T, site_ptr(CB, j), CB.dims[j], CB.dims[j + 1], mbase + moff[j], mdims[j], mdims[j + 1], d,
+                  (mp * row[j]) % d, (mp * row[n + j]) % d, nullptr, 0);
   const double2 v = E[0];
   __syncthreads();
   return v;
