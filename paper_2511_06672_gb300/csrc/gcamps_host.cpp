@@ -362,6 +362,8 @@ struct gcamps {
   int8_t* xz_dev = nullptr;
   double2* out_dev = nullptr;
   double* schmidt_dev = nullptr;
+  void* dense_dev = nullptr;           // dense readout: workspace, outputs, label (grown by larger registers)
+  size_t dense_cap = 0;
   double* score_dev = nullptr;         // gcamps_score_theta: outputs and scores (allocated by its first call)
   int* cnt_dev = nullptr;
   int* replay_dev = nullptr;           // [batch][kDecCap][2] recorded decisions to replay
@@ -763,6 +765,7 @@ void gcamps_destroy(gcamps_t* h) {
   if (h->ops_dev) cudaFree(h->ops_dev);
   if (h->begin_dev) cudaFree(h->begin_dev);
   if (h->schmidt_dev) cudaFree(h->schmidt_dev);
+  if (h->dense_dev) cudaFree(h->dense_dev);
   if (h->score_dev) cudaFree(h->score_dev);
   if (h->replay_dev) cudaFree(h->replay_dev);
   if (h->replay_n_dev) cudaFree(h->replay_n_dev);
@@ -1026,27 +1029,29 @@ static int statevector_impl(gcamps_t* h, int circuit, const int32_t* ys, long lo
     dim *= d;
     if (dim > (1LL << 20)) return fail(h, GCAMPS_EINVAL, "d^n above 2^20: dense readout not supported");
   }
-  const long long nbuf = dim * (long long)h->e.maxdim;
-  const size_t bytes = (size_t)(2 * nbuf + 3 * dim) * sizeof(double2) + (size_t)dim * (2 * sizeof(int) + n) + 256;
-  void* work = nullptr;
-  if (cudaMalloc(&work, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    return fail(h, GCAMPS_ENOMEM, "statevector workspace");
+  // the workspace (64 MB at 2^20 entries), the outputs and the label stay with the handle
+  const size_t work_bytes = (gcx::statevector_work(dim) + 255) / 256 * 256;
+  const size_t bytes = work_bytes + (size_t)dim * sizeof(double2) + 256;
+  if (bytes > h->dense_cap) {
+    if (h->dense_dev) cudaFree(h->dense_dev);   // idle: every readout waits for its result
+    h->dense_dev = nullptr;
+    h->dense_cap = 0;
+    if (cudaMalloc(&h->dense_dev, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(h, GCAMPS_ENOMEM, "statevector workspace");
+    }
+    h->dense_cap = bytes;
   }
-  int32_t* ys_dev = nullptr;
-  double2* out = nullptr;
-  cudaError_t ce = cudaMalloc(&out, (size_t)nys * sizeof(double2));
-  if (ce == cudaSuccess && ys) ce = cudaMalloc(&ys_dev, (size_t)nys * sizeof(int32_t));
-  if (ce == cudaSuccess && ys)
-    ce = cudaMemcpyAsync(ys_dev, ys, (size_t)nys * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream);
-  if (ce == cudaSuccess) ce = gcx::launch_statevector(h->e, circuit, out, dim, ys_dev, nys, work, h->stream);
+  char* base = (char*)h->dense_dev;
+  double2* out = (double2*)(base + work_bytes);
+  int32_t* ys_dev = ys ? (int32_t*)(base + work_bytes + (size_t)dim * sizeof(double2)) : nullptr;
+  cudaError_t ce = cudaSuccess;
+  if (ys) ce = cudaMemcpyAsync(ys_dev, ys, (size_t)nys * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream);
+  if (ce == cudaSuccess) ce = gcx::launch_statevector(h->e, circuit, out, dim, ys_dev, nys, base, h->stream);
   std::vector<double2> host((size_t)nys);
   if (ce == cudaSuccess)
     ce = cudaMemcpyAsync(host.data(), out, (size_t)nys * sizeof(double2), cudaMemcpyDeviceToHost, h->stream);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(h->stream);
-  cudaFree(work);
-  if (out) cudaFree(out);
-  if (ys_dev) cudaFree(ys_dev);
   if (ce != cudaSuccess) return cuda_fail(h, ce, "statevector");
   for (long long i = 0; i < nys; ++i) {
     re[i] = host[(size_t)i].x;
