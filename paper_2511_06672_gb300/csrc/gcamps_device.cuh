@@ -1048,8 +1048,12 @@ struct SmallSplit {
   int k;
   double disc;
 };
+// rank_one: M is likely of rank one (a class that the purity test chose): if what its largest column u leaves of the
+// others, |B - u u^H B|_F, is at most 1e-14 and cutoff of the norm, every other singular value is below the cutoff and
+// u, u^H B are its factors to rounding, without rotations (4 instead of 20-35 kcycles).
 __device__ __noinline__ SmallSplit svd_small(Smem& s, const Ctx& C, const double2* M, int rows, int cols, int cap,
-                                             bool renorm, double2* U, bool us, double2* Vh, bool vs) {
+                                             bool renorm, double2* U, bool us, double2* Vh, bool vs,
+                                             bool rank_one = false) {
   const Engine& e = *C.e;
   const bool tall = rows >= cols;
   const int m = tall ? rows : cols, n = tall ? cols : rows, L = m + n;
@@ -1065,9 +1069,73 @@ __device__ __noinline__ SmallSplit svd_small(Smem& s, const Ctx& C, const double
   for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x)
     s.z[(idx / n) * L + m + idx % n] = make_double2(idx / n == idx % n ? 1.0 : 0.0, 0.0);
   fro = block_sum(fro, s);
+  const int G = lanes_for(m), P = 32 / G;
+  if (rank_one) {
+    for (int j0 = warp; j0 < n; j0 += kWarps * P) {
+      const int j = j0 + kWarps * (lane / G);
+      double a = 0, b = 0;
+      if (j < n)
+        for (int r = lane & (G - 1); r < m; r += G) a += cabs2(s.z[j * L + r]);
+      group_sum2(a, b, G);
+      if (j < n && (lane & (G - 1)) == 0) s.zinv[j] = a;
+    }
+    __syncthreads();
+    int top = 0;
+    for (int j = 1; j < n; ++j)   // >= 0: ordered as integers
+      if (__double_as_longlong(s.zinv[j]) > __double_as_longlong(s.zinv[top])) top = j;
+    const double2* big = s.z + top * L;
+    const double inv = s.zinv[top] > 0.0 ? 1.0 / sqrt(s.zinv[top]) : 0.0;
+    for (int j0 = warp; j0 < n; j0 += kWarps * P) {
+      const int j = j0 + kWarps * (lane / G);
+      double wr = 0, wi = 0, res = 0, b = 0;
+      if (j < n)
+        for (int r = lane & (G - 1); r < m; r += G) {
+          const double2 x = big[r], y = s.z[j * L + r];
+          wr = fma(x.x, y.x, fma(x.y, y.y, wr));
+          wi = fma(x.x, y.y, fma(-x.y, y.x, wi));
+        }
+      group_sum2(wr, wi, G);
+      const double2 w = make_double2(wr * inv, wi * inv);   // u^H b_j
+      const double tr = w.x * inv, ti = w.y * inv;
+      if (j < n)
+        for (int r = lane & (G - 1); r < m; r += G) {
+          const double2 x = big[r], y = s.z[j * L + r];
+          const double dx = fma(-x.x, tr, fma(x.y, ti, y.x)), dy = fma(-x.x, ti, fma(-x.y, tr, y.y));
+          res = fma(dx, dx, fma(dy, dy, res));
+        }
+      group_sum2(res, b, G);
+      if (j < n && (lane & (G - 1)) == 0) {
+        s.zdiag[j] = w;
+        s.zbeta[j] = res;
+      }
+    }
+    __syncthreads();
+    double sig2 = 0, res = 0;   // every warp, the same sums
+    if (lane < n) {
+      sig2 = cabs2(s.zdiag[lane]);
+      res = s.zbeta[lane];
+    }
+    group_sum2(sig2, res, 32);
+    if (sig2 > 0.0 && res <= fmin(e.cutoff * e.cutoff, 1e-28) * sig2) {
+      const double sig = sqrt(sig2), isig = 1.0 / sig, out = renorm ? 1.0 : sig;   // the kept value, rescaled
+      const double fu = us ? out : 1.0, fv = vs ? out : 1.0;
+      for (int r = threadIdx.x; r < rows; r += blockDim.x)
+        U[r] = tall ? cscale(big[r], inv * fu) : cscale(cconj(s.zdiag[r]), isig * fu);
+      for (int c = threadIdx.x; c < cols; c += blockDim.x)
+        Vh[c] = tall ? cscale(s.zdiag[c], isig * fv) : cscale(cconj(big[c]), inv * fv);
+      if (threadIdx.x == 0) {
+        C.sing[0] = out;
+        C.stats[S_SVD] += 1;
+      }
+      SmallSplit f;
+      f.k = 1;
+      f.disc = res;
+      __syncthreads();
+      return f;
+    }
+  }
   const int sweeps = jacobi_small(s, m, n, fro, e.jacobi_cap);
   // column norms, G lanes a column
-  const int G = lanes_for(m), P = 32 / G;
   for (int j0 = warp; j0 < n; j0 += kWarps * P) {
     const int j = j0 + kWarps * (lane / G);
     double a = 0, b = 0;
@@ -3746,7 +3814,8 @@ __device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, b
   }
   Factor F;
   if (svd_fits(rows, cols)) {
-    const SmallSplit f = svd_small(s, C, theta, rows, cols, cap, true, site_ptr(C, i), !ltr, site_ptr(C, i + 1), ltr);
+    const SmallSplit f = svd_small(s, C, theta, rows, cols, cap, true, site_ptr(C, i), !ltr, site_ptr(C, i + 1), ltr,
+                                   kb != 0 && s.ival[7]);
     F.k = f.k;
     F.disc = f.disc;
   } else if (big) {
