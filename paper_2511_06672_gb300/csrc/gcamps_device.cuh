@@ -1873,6 +1873,12 @@ struct WarpGroup {
   static constexpr int n = 32;
   __device__ void sync() const { __syncwarp(); }
   __device__ double sum(double v) const { return warp_sum(v); }
+  // the sum when only the first `count` threads hold a value: the levels their lanes need
+  __device__ double sum_first(double v, int count) const {
+    for (int o = count > 16 ? 16 : (count > 8 ? 8 : (count > 4 ? 4 : 2)); o > 0; o >>= 1)
+      v += __shfl_xor_sync(0xffffffffu, v, o);
+    return __shfl_sync(0xffffffffu, v, 0);
+  }
   __device__ float sumf(float v) const { return warp_sum_f(v); }
   __device__ double bcast(double v) const { return __shfl_sync(0xffffffffu, v, 0); }
   // thread 0's v (after its memory writes) to every thread of the group
@@ -1909,6 +1915,7 @@ struct BlockGroup {
   int tid, n;
   __device__ void sync() const { __syncthreads(); }
   __device__ double sum(double v) const { return block_sum(v, *s); }
+  __device__ double sum_first(double v, int) const { return block_sum(v, *s); }
   __device__ float sumf(float v) const { return block_sum_f(v, *s); }
   __device__ double bcast(double v) const {
     __syncthreads();
@@ -1943,7 +1950,7 @@ __device__ void group_tridiag(const Grp& g, double2* A, int m, double* dg, doubl
     // hide a small tail (which, inside a degenerate eigenspace, moves eigenvalues at first order)
     double tail2 = 0;
     for (int i = 1 + g.tid; i < r; i += g.n) tail2 += cabs2(A[(long long)(k + 1 + i) * m + k]);
-    tail2 = g.sum(tail2);
+    tail2 = g.sum_first(tail2, r);
     // the step's scalars on thread 0 alone (every warp computing them would put each FP64 pipe through
     // them twice): |x0|, alpha = |x|, the reflector's head x0 + phase(x0) alpha, h = v^H v / 2; published
     // as 1 / h, or -1 for a column that is already reduced
@@ -1953,19 +1960,21 @@ __device__ void group_tridiag(const Grp& g, double2* A, int m, double* dg, doubl
       // |x0|^2 in the normal range: one reciprocal square root gives |x0| and the phase x0 / |x0| (each
       // within two units of the last place); outside it, hypot and unit_phase with their rescaling
       const double s0 = fma(x0.x, x0.x, x0.y * x0.y);
-      const bool fast = s0 > 0x1p-1000 && s0 < 0x1p+1000;
-      const double rs = fast ? rsqrt(s0) : 0.0;
+      const bool fast = s0 > 0x1p-900 && tail2 < 0x1p+900 && s0 < 0x1p+900;
+      const double rs = fast ? rsqrt_fast(s0) : 0.0;
       const double ax0 = fast ? s0 * rs : hypot(x0.x, x0.y);
       dg[k] = A[(long long)k * m + k].x;
       if (tail2 <= 1e-32 * fro2) {
         od[k] = ax0;
         pub = -1.0;
       } else {
-        const double alpha = sqrt(tail2 + ax0 * ax0);
+        const double a2 = tail2 + (fast ? s0 : ax0 * ax0);
+        const double alpha = fast ? a2 * rsqrt_fast(a2) : sqrt(a2);
         const double2 ph = fast ? make_double2(x0.x * rs, x0.y * rs) : unit_phase(x0);
         A[(long long)(k + 1) * m + k] = make_double2(x0.x + ph.x * alpha, x0.y + ph.y * alpha);
         od[k] = alpha;
-        pub = 1.0 / (alpha * (alpha + ax0));
+        const double h = fma(alpha, ax0, a2);
+        pub = fast ? rcp_fast(h) : 1.0 / h;
       }
     }
     const double hinv = g.publish(pub);
@@ -2016,7 +2025,7 @@ __device__ void group_tridiag(const Grp& g, double2* A, int m, double* dg, doubl
       const double2 v = A[(long long)(k + 1 + i) * m + k], p = A[(long long)k * m + k + 1 + i];
       kr += v.x * p.x + v.y * p.y;
     }
-    kr = g.sum(kr) * 0.5 * hinv;
+    kr = g.sum_first(kr, r) * 0.5 * hinv;
     g.sync();
     for (int i = g.tid; i < r; i += g.n) {
       const double2 v = A[(long long)(k + 1 + i) * m + k], p = A[(long long)k * m + k + 1 + i];
