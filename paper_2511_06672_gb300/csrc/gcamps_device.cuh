@@ -2255,6 +2255,11 @@ __device__ void tridiag_bisect(const Grp& g, const double* dg, double* od, int m
     for (int i = g.tid; i + 1 < m; i += g.n) od[i] = fmax(od[i] * od[i], e2min);
   }
   g.sync();
+  // The eigenvalues of a rank-deficient Gram that are zero to rounding: one count at 2^-51 span says how many lie
+  // below it, and 0 is within the accuracy for each.  (Two thirds of them on the benchmark circuits' bonds, where they
+  // also kept the Newton attempt below from verifying.)
+  const int m0 = fast ? sturm_count(D, E, m, 4.440892098500626e-16 * span) : 0, me = m - m0;
+  for (int i = g.tid; i < m0; i += g.n) ev[i] = 0.0;
   // Multisection: P lanes of a warp share eigenvalue j and count at P interior points of its
   // interval, which then shrinks by P + 1 per step (P as large as the group's warps allow).  All
   // lanes of a warp run the same number of steps (the group's outcome is combined by a ballot).
@@ -2268,7 +2273,7 @@ __device__ void tridiag_bisect(const Grp& g, const double* dg, double* od, int m
   {
     int best = 1 << 30;
     for (int p = 8; p >= 1; --p) {
-      const int pw = 32 / p, need = (m + pw - 1) / pw, passes = (need + nw - 1) / nw;
+      const int pw = 32 / p, need = (me + pw - 1) / pw, passes = (need + nw - 1) / nw;
       const int busiest = passes > 1 ? (nw + 3) / 4 : (need + 3) / 4;
       const int cost = passes * kIt64[p] * max(192 * busiest, 340);
       if (cost < best) {
@@ -2286,8 +2291,8 @@ __device__ void tridiag_bisect(const Grp& g, const double* dg, double* od, int m
   const int it32 = (int)ceil(24.0 / kLog2[P] - 1e-9);
   const int it64 = (int)ceil(33.0 / kLog2[P] - 1e-9);
   const int itfull = (int)ceil(50.0 / kLog2[P] - 1e-9);
-  for (int base = 0; base < m; base += nw * per_warp) {
-    const int jr = base + warp * per_warp + grp;
+  for (int base = 0; base < me; base += nw * per_warp) {
+    const int jr = m0 + base + warp * per_warp + grp;
     const bool active = grp < per_warp && jr < m;
     const int j = active ? jr : 0;
     double lo = gl, hi = gu;
