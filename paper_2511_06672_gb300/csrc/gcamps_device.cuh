@@ -188,7 +188,7 @@ __device__ __forceinline__ double rcp_fast(double a) {
 // One Clifford on (q0, q1) (q1 = q0 for one qudit): the exponents of its generator images, generator k's at
 // a[4 k .. 4 k + 3] in the order x_q0, z_q0, x_q1, z_q1, and their phases r; s = z(g_k) . x(g_l) for k <= l, in row
 // order; inv: the images of its inverse, 4 exponents and the phase each.
-constexpr int kGates = 64;   // gates on disjoint qudits are at most kMaxN / 2
+constexpr int kGates = kMaxN;   // gates on disjoint qudits
 struct GateTab {
   uint8_t a[16], r[4], s[10], inv[20];
   uint8_t q0, q1, ng;        // ng: generators, 2 or 4
@@ -225,7 +225,7 @@ struct Smem {
       GateTab gate[kGates];
       int ph[2 * kMaxN];          // phase each row gains
       int first[kMaxN];           // first gate of the window on a qudit
-      int nlead;                  // gates before the first that shares a qudit with an earlier one
+      int nlead;                  // gates taken this round
     };
   };
   float redh[2][kWarps / 2];    // partial sums of the half-CTA groups
@@ -579,30 +579,38 @@ __device__ void tableau_gates(Smem& s, const Ctx& C, int ng, uint8_t* cx, uint8_
 }
 
 // C <- G C (Sec. 3, top loop of Fig. 3) for count Clifford gates in order: forward rows conjugated by G, the rows of
-// the inverse tableau for G's sites replaced by products of old rows.  Each step takes the longest run of gates on
-// disjoint qudits.
+// the inverse tableau for G's sites replaced by products of old rows.  A window of kThreads gates, a thread each; each
+// round takes every gate that is the first one left on all of its qudits (the gates left before it share no qudit
+// with it, so it commutes with them): as many rounds as the window is deep, whatever the order of the list.
 template <int D>
 __device__ void clifford_steps(Smem& s, const Ctx& C, const gcamps_op* ops, int count) {
   const int tid = threadIdx.x;
-  for (int p = 0; p < count;) {
-    const int w = min(count - p, kGates);
-    for (int q = tid; q < C.n; q += blockDim.x) s.first[q] = kGates;
-    if (tid == 0) s.nlead = w;
-    __syncthreads();
+  for (int p = 0; p < count; p += kThreads) {
+    const int w = min(count - p, kThreads);
     int q0 = 0, q1 = -1;
-    if (tid < w) {
+    bool left = tid < w;
+    if (left) {
       q0 = ops[p + tid].q0;
       q1 = ops[p + tid].q1;
-      atomicMin(&s.first[q0], tid);
-      if (q1 >= 0) atomicMin(&s.first[q1], tid);
     }
-    __syncthreads();
-    if (tid < w && (s.first[q0] < tid || (q1 >= 0 && s.first[q1] < tid))) atomicMin(&s.nlead, tid);
-    __syncthreads();
-    const int ng = s.nlead;
-    if (tid < ng) gate_table<D>(s.gate[tid], ops[p + tid].img, q0, q1);
-    tableau_gates<D>(s, C, ng, C.fx, C.fr, C.ix, C.ir);
-    p += ng;
+    for (int done = 0; done < w;) {
+      for (int q = tid; q < C.n; q += blockDim.x) s.first[q] = kThreads;
+      if (tid == 0) s.nlead = 0;
+      __syncthreads();
+      if (left) {
+        atomicMin(&s.first[q0], tid);
+        if (q1 >= 0) atomicMin(&s.first[q1], tid);
+      }
+      __syncthreads();
+      if (left && s.first[q0] == tid && (q1 < 0 || s.first[q1] == tid)) {
+        gate_table<D>(s.gate[atomicAdd(&s.nlead, 1)], ops[p + tid].img, q0, q1);   // at most n gates
+        left = false;
+      }
+      __syncthreads();
+      const int ng = s.nlead;
+      tableau_gates<D>(s, C, ng, C.fx, C.fr, C.ix, C.ir);
+      done += ng;
+    }
   }
 }
 __device__ __noinline__ void apply_cliffords(Smem& s, const Ctx& C, const gcamps_op* ops, int count) {
