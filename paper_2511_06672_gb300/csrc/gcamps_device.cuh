@@ -4023,23 +4023,23 @@ __device__ void conj_weyl(Smem& s, const Ctx& C, const int8_t* xz, int* acc_x, i
   __syncthreads();
 }
 
-// store(o, sum_{k < K} term(o)(k)) for o < count on the CTA: P lanes share a sum, P chosen for the busiest FP64 pipe
-// (passes x warps a pipe x (4 ceil(K / P) multiply-adds + 2 log2 P adds)).
+// store(o, sum_{k < K} term(o)(k)) for o < count on a group of nt threads (whole warps): P lanes share a sum, P chosen
+// for the busiest FP64 pipe (passes x warps a pipe x (4 ceil(K / P) multiply-adds + 2 log2 P adds)).
 template <class Term, class Store>
-__device__ __forceinline__ void split_sums(int count, int K, Term term, Store store) {
+__device__ __forceinline__ void split_sums(int tid, int nt, int count, int K, Term term, Store store) {
   int P = 1, best = 1 << 30;
   for (int q = 1, lg = 0; q <= 32 && (q == 1 || q <= K); q *= 2, ++lg) {
-    const int outs = kThreads / q, passes = (count + outs - 1) / outs;
-    const int warps = min(kWarps, (min(count, outs) * q + 31) / 32);
+    const int outs = nt / q, passes = (count + outs - 1) / outs;
+    const int warps = min(nt / 32, (min(count, outs) * q + 31) / 32);
     const int cost = passes * ((warps + 3) / 4) * (4 * ((K + q - 1) / q) + 2 * lg);
     if (cost < best) {
       best = cost;
       P = q;
     }
   }
-  const int outs = kThreads / P, c = threadIdx.x & (P - 1);
+  const int outs = nt / P, c = tid & (P - 1);
   for (int base = 0; base < count; base += outs) {
-    const int o = base + (int)threadIdx.x / P;
+    const int o = base + tid / P;
     double2 acc = cz();
     if (o < count) {
       const auto t = term(o);
@@ -4055,12 +4055,11 @@ __device__ __forceinline__ void split_sums(int count, int K, Term term, Store st
 
 // One site of <A| X^x Z^z |M>: E[a, a'] (bl x ml) becomes E'[b, b'] (br x mr), in place, through
 // T[a, s, b'] = sum_{a'} E[a, a'] omega^{z (s - x)} M[a', s - x, b'],  E'[b, b'] = sum_{a, s} conj(A[a, s, b]) T[a, s, b'].
-// next: the following site's tensors, fetched towards the SM meanwhile (null: none).
-__device__ void transfer_site(Smem& s, double2* E, double2* T, const double2* A, int bl, int br, const double2* M, int ml,
-                              int mr, int d, int x, int z, const double2* next, int next_count) {
-  if (next && (int)threadIdx.x * 8 < next_count)
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(next + threadIdx.x * 8));
-  split_sums(bl * d * mr, ml,
+// Grp: a CTA or half of one.
+template <class Grp>
+__device__ void transfer_site(const Grp& g, const Smem& s, double2* E, double2* T, const double2* A, int bl, int br,
+                              const double2* M, int ml, int mr, int d, int x, int z) {
+  split_sums(g.tid, g.n, bl * d * mr, ml,
              [&](int o) {
                const int bp = o % mr, sd = (o / mr) % d, a = o / (mr * d);
                const int sp = sd >= x ? sd - x : sd - x + d;
@@ -4073,15 +4072,43 @@ __device__ void transfer_site(Smem& s, double2* E, double2* T, const double2* A,
                const int ph = (2 * z * sp) % (2 * d);
                T[o] = ph ? cmul(s.tau[ph], acc) : acc;
              });
-  __syncthreads();
-  split_sums(br * mr, bl * d,
+  g.sync();
+  split_sums(g.tid, g.n, br * mr, bl * d,
              [&](int o) {
                const double2* a = A + o / mr;
                const double2* t = T + o % mr;
                return [=](int k, double2 acc) { return cfmac(a[(long long)k * br], t[(long long)k * mr], acc); };
              },
              [&](int o, double2 acc) { E[o] = acc; });
-  __syncthreads();
+  g.sync();
+}
+// The same from the right for one state: F[b, b'] (cr x cr) becomes F'[a, a'] (cl x cl), through
+// T[s, b, a'] = sum_{b'} omega^{z (s - x)} A[a', s - x, b'] F[b, b'],  F'[a, a'] = sum_{s, b} conj(A[a, s, b]) T[s, b, a'].
+template <class Grp>
+__device__ void transfer_site_left(const Grp& g, const Smem& s, double2* F, double2* T, const double2* A, int cl, int cr,
+                                   int d, int x, int z) {
+  split_sums(g.tid, g.n, d * cr * cl, cr,
+             [&](int o) {
+               const int ap = o % cl, b = (o / cl) % cr, sd = o / (cl * cr);
+               const int sp = sd >= x ? sd - x : sd - x + d;
+               const double2* f = F + (long long)b * cr;
+               const double2* m = A + ((long long)ap * d + sp) * cr;
+               return [=](int k, double2 acc) { return cfma(f[k], m[k], acc); };
+             },
+             [&](int o, double2 acc) {
+               const int sd = o / (cl * cr), sp = sd >= x ? sd - x : sd - x + d;
+               const int ph = (2 * z * sp) % (2 * d);
+               T[o] = ph ? cmul(s.tau[ph], acc) : acc;
+             });
+  g.sync();
+  split_sums(g.tid, g.n, cl * cl, d * cr,
+             [&](int o) {
+               const double2* a = A + (long long)(o / cl) * d * cr;
+               const double2* t = T + o % cl;
+               return [=](int k, double2 acc) { return cfmac(a[k], t[(long long)k * cl], acc); };
+             },
+             [&](int o, double2 acc) { F[o] = acc; });
+  g.sync();
 }
 // Shared memory for E and T where every bond of both states allows it: bra bond dimensions ba, ket ones bk.
 constexpr int kTransferE = 200;   // E's part of s.z

@@ -18,9 +18,10 @@ __device__ double2 overlap_weyl(Smem& s, const Ctx& CB, const double2* mbase, co
   double2* T = fits ? s.z + kTransferE : CB.scr + e.sl.tmp;
   if (threadIdx.x == 0) E[0] = make_double2(1.0, 0.0);
   __syncthreads();
+  const BlockGroup g{&s, (int)threadIdx.x, (int)blockDim.x};
   for (int j = 0; j < n; ++j)
-    transfer_site(s, E, T, site_ptr(CB, j), CB.dims[j], CB.dims[j + 1], mbase + moff[j], mdims[j], mdims[j + 1], d,
-                  (mp * row[j]) % d, (mp * row[n + j]) % d, nullptr, 0);
+    transfer_site(g, s, E, T, site_ptr(CB, j), CB.dims[j], CB.dims[j + 1], mbase + moff[j], mdims[j], mdims[j + 1], d,
+                  (mp * row[j]) % d, (mp * row[n + j]) % d);
   const double2 v = E[0];
   __syncthreads();
   return v;

@@ -402,12 +402,8 @@ long long sat_pow(int d, int k, long long cap) {
   return v;
 }
 
-int device_status(gcamps_t* h) {
-  std::vector<int> meta((size_t)h->e.batch * gcx::M_COUNT);
-  cudaError_t e = cudaMemcpyAsync(meta.data(), h->e.meta, meta.size() * sizeof(int), cudaMemcpyDeviceToHost,
-                                  h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e, "device status");
+// The code and message of the first failed circuit among the status words.
+int check_status(gcamps_t* h, const int* meta) {
   for (int c = 0; c < h->e.batch; ++c) {
     const int* mc = &meta[(size_t)c * gcx::M_COUNT];
     const int s = mc[gcx::M_STATUS];
@@ -422,6 +418,15 @@ int device_status(gcamps_t* h) {
     }
   }
   return GCAMPS_OK;
+}
+
+int device_status(gcamps_t* h) {
+  std::vector<int> meta((size_t)h->e.batch * gcx::M_COUNT);
+  cudaError_t e = cudaMemcpyAsync(meta.data(), h->e.meta, meta.size() * sizeof(int), cudaMemcpyDeviceToHost,
+                                  h->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  if (e != cudaSuccess) return cuda_fail(h, e, "device status");
+  return check_status(h, meta.data());
 }
 
 }  // namespace
@@ -679,7 +684,9 @@ int gcamps_create_batch_uneven(int batch, const int32_t* nqs, int d, int chi_max
   const size_t o_grad = bytes;
   if (snap) bytes = align(bytes + (size_t)opts.snapshot_max_gates * 4 * sizeof(double));
   const size_t o_aux = bytes;
-  bytes = align(bytes + (size_t)(gcx::kMaxN * 2 + 64) + 4096);
+  // a string's exponents | a value and the status words behind it | a count
+  const size_t out_bytes = align(sizeof(double2) + (size_t)batch * gcx::M_COUNT * sizeof(int));
+  bytes = align(bytes + align(gcx::kMaxN * 2) + out_bytes + 64);
   if (opts.cuda_stream) {
     h->stream = (cudaStream_t)opts.cuda_stream;
   } else {
@@ -727,7 +734,7 @@ int gcamps_create_batch_uneven(int batch, const int32_t* nqs, int d, int chi_max
   e.candImg = (const int32_t*)(base + o_candI);
   h->xz_dev = (int8_t*)(base + o_aux);
   h->out_dev = (double2*)(base + o_aux + align(gcx::kMaxN * 2));
-  h->cnt_dev = (int*)(h->out_dev + 2);
+  h->cnt_dev = (int*)(base + o_aux + align(gcx::kMaxN * 2) + out_bytes);
   cudaError_t ce = cudaMemcpyAsync((void*)e.site_off, h->site_off.data(), h->site_off.size() * sizeof(long long),
                                    cudaMemcpyHostToDevice, h->stream);
   if (ce == cudaSuccess)
@@ -965,12 +972,14 @@ int gcamps_batch_expect_weyl(gcamps_t* h, int circuit, const int32_t* x, const i
   }
   GC_CUDA(h, cudaMemcpyAsync(h->xz_dev, xz.data(), 2 * n, cudaMemcpyHostToDevice, h->stream));
   GC_CUDA(h, gcx::launch_expect(h->e, circuit, h->xz_dev, h->out_dev, h->stream));
-  double2 r;
-  GC_CUDA(h, cudaMemcpyAsync(&r, h->out_dev, sizeof r, cudaMemcpyDeviceToHost, h->stream));
+  // the value and, right behind it, the circuits' status words (k_expect puts them there): one copy, one wait
+  std::vector<double> r(2 + ((size_t)h->e.batch * gcx::M_COUNT * sizeof(int) + 7) / 8);
+  GC_CUDA(h, cudaMemcpyAsync(r.data(), h->out_dev, 2 * sizeof(double) + (size_t)h->e.batch * gcx::M_COUNT * sizeof(int),
+                             cudaMemcpyDeviceToHost, h->stream));
   GC_CUDA(h, cudaStreamSynchronize(h->stream));
-  *re = r.x;
-  *im = r.y;
-  return device_status(h);
+  *re = r[0];
+  *im = r[1];
+  return check_status(h, reinterpret_cast<const int*>(r.data() + 2));
 }
 
 int gcamps_expect_gradient(gcamps_t* h, int circuit, const int32_t* x, const int32_t* z, double* value,
@@ -1086,15 +1095,23 @@ int gcamps_batch_amplitude(gcamps_t* h, int circuit, const int32_t* digits, doub
   return statevector_impl(h, circuit, &yy, 1, re, im);
 }
 
+// Exponents and phases of the tableau at t (device memory, back to back): one copy.
+static int copy_tableau(gcamps_t* h, const uint8_t* t, int n, uint8_t* exps, uint8_t* phase) {
+  const size_t ne = (size_t)4 * n * n, np = (size_t)2 * n;
+  std::vector<uint8_t> both(ne + np);
+  GC_CUDA(h, cudaMemcpyAsync(both.data(), t, ne + np, cudaMemcpyDeviceToHost, h->stream));
+  const int rc = device_status(h);   // waits
+  if (exps) std::memcpy(exps, both.data(), ne);
+  if (phase) std::memcpy(phase, both.data() + ne, np);
+  return rc;
+}
+
 int gcamps_batch_get_tableau(gcamps_t* h, int circuit, uint8_t* exps, uint8_t* phase) {
   int rc = check_circuit(h, circuit);
   if (rc) return rc;
   const int n = h->nq[circuit];
   const uint8_t* t = h->e.tab + (long long)circuit * h->e.tab_stride;
-  if (exps) GC_CUDA(h, cudaMemcpyAsync(exps, t, 4 * n * n, cudaMemcpyDeviceToHost, h->stream));
-  if (phase) GC_CUDA(h, cudaMemcpyAsync(phase, t + 4 * n * n, 2 * n, cudaMemcpyDeviceToHost, h->stream));
-  GC_CUDA(h, cudaStreamSynchronize(h->stream));
-  return device_status(h);
+  return copy_tableau(h, t, n, exps, phase);
 }
 
 int gcamps_get_inverse_tableau(gcamps_t* h, int circuit, uint8_t* exps, uint8_t* phase) {
@@ -1102,10 +1119,7 @@ int gcamps_get_inverse_tableau(gcamps_t* h, int circuit, uint8_t* exps, uint8_t*
   if (rc) return rc;
   const int n = h->nq[circuit];
   const uint8_t* t = h->e.tab + (long long)circuit * h->e.tab_stride + 4 * n * n + 2 * n;
-  if (exps) GC_CUDA(h, cudaMemcpyAsync(exps, t, 4 * n * n, cudaMemcpyDeviceToHost, h->stream));
-  if (phase) GC_CUDA(h, cudaMemcpyAsync(phase, t + 4 * n * n, 2 * n, cudaMemcpyDeviceToHost, h->stream));
-  GC_CUDA(h, cudaStreamSynchronize(h->stream));
-  return device_status(h);
+  return copy_tableau(h, t, n, exps, phase);
 }
 
 int gcamps_batch_get_bond_dims(gcamps_t* h, int circuit, int32_t* chi) {
@@ -1113,12 +1127,14 @@ int gcamps_batch_get_bond_dims(gcamps_t* h, int circuit, int32_t* chi) {
   if (rc) return rc;
   if (!chi) return fail(h, GCAMPS_EINVAL, "null output");
   const int n = h->nq[circuit];
-  std::vector<int> dims(n + 1);
-  GC_CUDA(h, cudaMemcpyAsync(dims.data(), h->e.dims + (long long)circuit * (h->e.n + 1), (n + 1) * sizeof(int),
-                             cudaMemcpyDeviceToHost, h->stream));
+  // the circuit's bond dimensions up to the status words, which follow those of the last circuit: one copy, one wait
+  const int* first = h->e.dims + (long long)circuit * (h->e.n + 1);
+  const size_t upto = (const char*)(h->e.meta + (size_t)h->e.batch * gcx::M_COUNT) - (const char*)first;
+  std::vector<int> dims(upto / sizeof(int));
+  GC_CUDA(h, cudaMemcpyAsync(dims.data(), first, upto, cudaMemcpyDeviceToHost, h->stream));
   GC_CUDA(h, cudaStreamSynchronize(h->stream));
   for (int j = 0; j < n - 1; ++j) chi[j] = dims[j + 1];
-  return device_status(h);
+  return check_status(h, dims.data() + (h->e.meta - first));
 }
 
 // The single-circuit forms of the contract (circuit 0 of the handle).
