@@ -1162,11 +1162,14 @@ __device__ __noinline__ SmallSplit svd_small(Smem& s, const Ctx& C, const double
       const long long ki = __shfl_sync(0xffffffffu, key, i);
       rank += (ki > key) || (ki == key && i < lane);
     }
-    const double v = lane < n ? sqrt(v2) : 0.0;
+    const bool normal = v2 > 0x1p-900 && v2 < 0x1p+900;
+    const double iv = normal ? rsqrt_fast(v2) : (v2 > 0.0 ? 1.0 / sqrt(v2) : 0.0);
+    const double v = normal ? v2 * iv : sqrt(v2);
     __syncwarp();
     if (lane < n) {
       s.zperm[rank] = lane;
       s.zs[rank] = v;
+      s.zinv[rank] = iv;
     }
     __syncwarp();
     const double sv = lane < n ? s.zs[lane] : 0.0;
@@ -1178,7 +1181,6 @@ __device__ __noinline__ SmallSplit svd_small(Smem& s, const Ctx& C, const double
     group_sum2(kept, drop, 32);
     const double scale = (renorm && kept > 0) ? 1.0 / sqrt(kept) : 1.0;
     if (lane < n) {
-      s.zinv[lane] = sv > 0.0 ? 1.0 / sv : 0.0;
       s.zs[lane] = sv * scale;
       C.sing[lane] = lane < k ? sv * scale : sv;
     }
@@ -2019,6 +2021,7 @@ __device__ void group_tridiag(const Grp& g, double2* A, int m, double* dg, doubl
       double2 acc = cz();
       if (i < r) {
         const double2* arow = A + (long long)(k + 1 + i) * m + (k + 1);
+#pragma unroll 2
         for (int j = c; j < r; j += kc) acc = cfma(arow[j], A[(long long)(k + 1 + j) * m + k], acc);
       }
       for (int o = kc >> 1; o > 0; o >>= 1) {
@@ -2377,6 +2380,26 @@ __device__ void tridiag_bisect(const Grp& g, const double* dg, double* od, int m
           if (active && pidx == 0) ev[j] = x;
           continue;
         }
+        // a cluster that rounding spreads past tol fails there (most of the failures: the spectra are highly
+        // degenerate); its eigenvalues lie within 64 tol all the same, which two counts confirm, and 7 halvings
+        // finish instead of 33
+        const double wide = 64.0 * tol;
+        if (P == 1) {
+          if (active && !bad) {
+            vlo = sturm_count(D, E, m, x - wide);
+            vhi = sturm_count(D, E, m, x + wide);
+          }
+        } else {
+          int c = 0;
+          if (active && pidx < 2) c = sturm_count(D, E, m, pidx == 0 ? x - wide : x + wide);
+          vlo = __shfl_sync(0xffffffffu, c, g0);
+          vhi = __shfl_sync(0xffffffffu, c, g0 + 1);
+        }
+        if (__all_sync(0xffffffffu, !active || (!bad && vlo <= j && vhi > j))) {
+          lo = x - wide;
+          hi = x + wide;
+          nit = (int)ceil(7.0 / kLog2[P] - 1e-9);
+        }
       }
     }
     for (int it = 0; it < nit; ++it) {
@@ -2474,7 +2497,8 @@ __device__ Score score_class(const Grp& g, const Ctx& C, const double2* theta, i
     const double2* q = Q + (sd * d + t) * dd;
     const double2* th = theta + (long long)a * dd * cr + b;
     double2 acc = cz();
-    for (int u = 0; u < dd; ++u) acc = cfma(q[u], th[(long long)u * cr], acc);
+#pragma unroll 3
+    for (int u = 0; u < dd; ++u) acc = cfma(q[u], th[u * cr], acc);
     tp[idx] = acc;
   }
   g.sync();
@@ -2487,8 +2511,10 @@ __device__ Score score_class(const Grp& g, const Ctx& C, const double2* theta, i
     if (rows <= cols) {
       const double2* ri = tp + (long long)i * cols;
       const double2* rj = tp + (long long)j * cols;
+#pragma unroll 4
       for (int c = 0; c < cols; ++c) acc = cfmac(rj[c], ri[c], acc);   // sum_c ri conj(rj)
     } else {
+#pragma unroll 4
       for (int r = 0; r < rows; ++r) acc = cfmac(tp[(long long)r * cols + i], tp[(long long)r * cols + j], acc);
     }
     G[(long long)i * m + j] = acc;
@@ -3417,11 +3443,9 @@ __device__ int select_class(Smem& s, Smem* lead, const Ctx& C, const double2* th
   // The von Neumann score prunes with FP32 estimates whose error bound depends on the shape only: the leader
   // computes it once, published with the FP32 copy of theta by the barrier below.
   const bool est_kind = prune && kind == 0;
-  if (leader && threadIdx.x == 0) {
-    s.ival[6] = 0;
-    if (est_kind) s.dval[3] = vn_est_bound(d, m, rows < cols ? cols : rows);
-  }
-  if (prune) {   // FP32 copy of theta for the screen, shared by the cluster
+  if (leader && threadIdx.x == 0) s.ival[6] = 0;
+  if (prune && !search) {   // FP32 copy of theta for the screen, shared by the cluster; a visit publishes its own
+    if (leader && threadIdx.x == 0 && est_kind) s.dval[3] = vn_est_bound(d, m, rows < cols ? cols : rows);
     if (leader && !C.known)
       for (int i = threadIdx.x; i < rows * cols; i += blockDim.x)
         C.th32[i] = make_float2((float)theta[i].x, (float)theta[i].y);
@@ -3741,8 +3765,12 @@ __device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, b
     end_visit(C, m, tv);
     return;
   }
+  // theta, and what the scoring reads of it: its FP32 copy and the estimates' error bound
   block_matmul(theta, site_ptr(C, i), site_ptr(C, i + 1), rows, chim, cols);
+  for (int idx = threadIdx.x; idx < rows * cols; idx += blockDim.x)   // block_matmul's own entries
+    C.th32[idx] = make_float2((float)theta[idx].x, (float)theta[idx].y);
   if (threadIdx.x == 0) {
+    s.dval[3] = vn_est_bound(d, m, rows < cols ? cols : rows);
     s.rank0 = -1;
     s.vbond = i;
     s.ival[7] = 0;   // 1: the purity test decided
