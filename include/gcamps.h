@@ -79,12 +79,14 @@ typedef struct {
   int64_t t_gates;            /* non-Clifford gates applied                                 */
   int64_t clifford_gates;     /* Clifford gates applied to the tableau                      */
   int64_t bonds_visited;      /* disentangler bond visits                                   */
-  int64_t candidates_scored;  /* (bond, class) entanglement scores evaluated                */
+  int64_t candidates_scored;  /* (bond, class) pairs the search covered: K per bond visit,  */
+                              /* whether scored or known not to change the decision         */
   int64_t accepted;           /* disentanglers applied                                      */
   int64_t sweeps;             /* disentangling sweeps                                       */
-  int64_t vn_evaluations;     /* exact (FP64) von Neumann entropies computed; the other     */
-                              /* classes were excluded by the Renyi-2 lower bound S2 <= S_vN */
-                              /* or by their FP32 estimate's error bound                    */
+  int64_t vn_evaluations;     /* exact (FP64) scores computed (entropies, or the S2 of the  */
+                              /* purity test); the other classes were excluded by the       */
+                              /* Renyi-2 lower bound S2 <= S_vN or by their FP32 estimate's  */
+                              /* error bound, or the visit's decision was known without them */
   int64_t svd_calls;          /* truncating SVDs (one-sided Jacobi)                         */
   int64_t jacobi_sweeps;      /* Jacobi sweeps over all SVDs                                */
   int64_t jacobi_max_sweeps;  /* most sweeps one SVD needed                                 */
@@ -320,7 +322,7 @@ int gcamps_overlap(gcamps_t* h1, int circuit1, gcamps_t* h2, int circuit2, doubl
  *   [0] Clifford tableau updates          [1] non-Clifford steps (MPO apply and recompression)
  *   [2] centre moves before a sweep       [3] forming theta at a bond visit
  *   [4] FP32 Renyi-2 screen of every class [5] FP32 von Neumann estimates (their bounds)
- *   [6] exact FP64 class evaluations       [7] the decision
+ *   [6] exact FP64 class evaluations and the purity test   [7] the decision
  *   [8] applying the chosen class and folding it into the tableau
  *   [9] truncated SVD splits               [10] QR centre moves after a visit that applies nothing
  *   [12 + b] bond visits, [17 + b] their cycles, [22 + b] their exact evaluations, [27 + b] their FP32
@@ -338,7 +340,8 @@ int gcamps_get_profile(gcamps_t* h, int circuit, int64_t* out, int32_t cap, int3
  * FP64 where evaluated[k] = 1, else the FP32 screening value, within 4 eta sqrt(m) + 4 eta of the exact
  * one with eta < 3 (d^3 + 6 d + max side) 2^-24), vn[k] (von Neumann entropy, valid where
  * evaluated[k] = 1 except for classes scored by Renyi-2 alone under score_kind 1, which read NaN;
- * the bounds excluded the others);
+ * the bounds excluded the others; where the classes that make theta a product across the bond decided the
+ * visit, those are the evaluated ones and their vn is their S2, within tie_tol / 2 of the entropy);
  * K = gcamps_num_candidates(d) entries each; any pointer may be NULL. */
 int gcamps_get_last_scores(gcamps_t* h, int circuit, double* s2, double* vn, uint8_t* evaluated);
 /* Two-site tensor theta scored at the last bond visit (Sec. 3): shape[0..1] = (chi_l, chi_r); theta receives the

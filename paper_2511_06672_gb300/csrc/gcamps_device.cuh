@@ -249,8 +249,8 @@ struct Smem {
   int npure, pure;            // select_class: classes of the purity test, and whether it decided (leader)
   int vbond;                  // bond of the visit the cluster serves next, -1 to leave the sweeps (leader)
   uint8_t clean[kMaxN];       // bond b: the state around it is the one its last visit left (leader, disentangle)
-  // the leader's counters of the launch (load_counters): one thread adds to them several times per visit, which
-  // in global memory took about 10 of the 200 kcycles of a small visit
+  // the leader's counters of the launch (load_counters): one thread adds to them several times per visit, and the
+  // others wait for it (in global memory the decision phase of a small visit took 4.9 kcycles, here 1.4)
   long long stats[S_COUNT];
   long long prof[P_COUNT];
   double dstats[kDStats];
@@ -420,7 +420,7 @@ __device__ void block_matmul(double2* Cm, const double2* A, const double2* B, in
 // Gates on disjoint qudits commute and touch disjoint columns (conjugated rows) or rows (row products) of a tableau,
 // so a whole brickwork layer goes at once: a thread per (row, gate), a warp per gate's rows, four barriers.  Gate by
 // gate, each with a d^4-entry table, a layer of 48 gates on 96 qutrits took 650 kcycles, bound by the barriers
-// and by reads of a few bytes each.
+// and by reads of a few bytes each; together they take 63.
 
 // Phase (units of tau) of prod_k (tau^{r_k} W(g_k))^{v_k}, the product taken in the order of k with the Weyl rule
 // (tau^r W(a)) (tau^r' W(b)) = tau^{r + r' + 2 z(a) . x(b)} W(a + b), s as in GateTab.
@@ -967,9 +967,9 @@ __device__ __forceinline__ bool svd_fits(int rows, int cols) {
 // The rotations of jacobi_orthogonalize on the columns of s.z, each the m entries of B over the n of W (stride m + n),
 // so that one pass rotates both.  Rounds: for odd n the pairs with i + j = 2 round (mod n), (n - 1) / 2 of them and
 // no idle slot; for even n the round-robin of jacobi_orthogonalize.  The rotation's cosine and sine come from two
-// reciprocal square roots: with r = 1 / sqrt(1 + zeta^2), c^2 = (1 + |zeta| r) / 2 and s c = r / 2.  About 40 FP64
-// instructions a pair instead of 130; a 9-column sweep takes 30 instead of 90 kcycles.  n = 2, 3 has one pair a
-// round: one warp does it without CTA barriers.
+// reciprocal square roots: with r = 1 / sqrt(1 + zeta^2), c^2 = (1 + |zeta| r) / 2 and s c = r / 2.  About 55 FP64
+// instructions a pair instead of 130.  Splits of the visits with m <= 9 took 57 kcycles on average before and 32 with
+// this (qutrits; qubits 20 and 9.6).  n = 2, 3 has one pair a round: one warp does it without CTA barriers.
 __device__ int jacobi_small(Smem& s, int m, int n, double fro, int max_sweeps) {
   if (n <= 1) return 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1058,7 +1058,8 @@ struct SmallSplit {
 };
 // rank_one: M is likely of rank one (a class that the purity test chose): if what its largest column u leaves of the
 // others, |B - u u^H B|_F, is at most 1e-14 and cutoff of the norm, every other singular value is below the cutoff and
-// u, u^H B are its factors to rounding, without rotations (4 instead of 20-35 kcycles).
+// u, u^H B are its factors to rounding, without rotations (a third fewer Jacobi sweeps per circuit; splits at m <= 9
+// 32 -> 29 kcycles on average, 18 -> 14.5 in a batch whose visits mostly end in products).
 __device__ __noinline__ SmallSplit svd_small(Smem& s, const Ctx& C, const double2* M, int rows, int cols, int cap,
                                              bool renorm, double2* U, bool us, double2* Vh, bool vs,
                                              bool rank_one = false) {
@@ -1220,7 +1221,7 @@ __device__ __noinline__ SmallSplit svd_small(Smem& s, const Ctx& C, const double
 // block_qr's reflectors: R's part above the diagonal stays in s.z, its diagonal goes to s.zdiag, Q (m x k) follows
 // the matrix.  One barrier a step: the group that owns the next column takes that column's norm and reflector
 // right after its update, the other columns' groups meanwhile finish theirs; Q's columns need none (column c is
-// H_0 .. H_c e_c).  9 x 3: 12 instead of 25 kcycles.
+// H_0 .. H_c e_c).  With svd_small, the MPO steps of a 32-qutrit circuit went from 64 to 33 Mcycles.
 __device__ __forceinline__ bool qr_fits(int m, int n) { return n < kZCols && m * n + m * (m < n ? m : n) <= kZ; }
 
 __device__ int qr_small(Smem& s, int m, int n, double fro) {
@@ -3452,8 +3453,8 @@ __device__ int select_class(Smem& s, Smem* lead, const Ctx& C, const double2* th
     cluster_sync();
   }
   // First the classes that make theta' a product across the bond (about 80 % of the visits that apply a class on
-  // the benchmark circuits): the FP32 screen finds them, their FP64 S2 settles them (pure_choice).  A Gram
-  // instead of a Gram, its reduction and its eigenvalues: 15 instead of 68 kcycles a class at m = 9.
+  // the benchmark circuits): the FP32 screen finds them, their FP64 S2 settles them (pure_choice).  A class then
+  // takes its Gram (11 kcycles at m = 9) instead of its Gram, reduction, eigenvalues and entropy (68).
   const bool screened = search && est_kind && e.tie_tol >= 1e-12 && e.tie_tol <= 1e-4;
   if (screened) {
     score_classes(s, lead, C, theta, cl, cr, nullptr, C.K, kScreen);
@@ -3741,7 +3742,8 @@ __device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, b
     C.prof[P_CURB] = 1 + prof_bucket(m);
     C.prof[P_VISITS + prof_bucket(m)] += 1;
   }
-  // Two kinds of visit apply nothing whatever the classes' scores (60 % of the visits on the benchmark circuits):
+  // Two kinds of visit apply nothing whatever the classes' scores (half of the visits on the benchmark circuits; with
+  // the purity test a visit's mean fell from 197 to 137 kcycles, qubits 113 to 67):
   // a bond of dimension 1 has entropy 0, which no class lowers; and around a clean bond nothing has changed since
   // its last visit but unitaries on one side of the pair's two sites, which leave every class's score as it was
   // (the classes of Q theta are those of theta, so after applying the best one the identity is the best).  The
@@ -4021,8 +4023,8 @@ __device__ void run_op(Smem& s, Smem* lead, const Ctx& C, const gcamps_op& op, i
 // P' = C^dag W C for W = (x)_j X_j^{x_j} Z_j^{z_j} (xz = x | z): the inverse-tableau rows multiplied in
 // the order of W with the Weyl product rule; exponents into acc_x, acc_z and the phase (units of tau)
 // into *acc_r, all in shared memory.  A thread per column: the phase is a sum over columns of (z so far) x (row's x),
-// so the columns need each other only in its total (the rows one by one, each with a CTA-wide sum, took 100 kcycles
-// at n = 32).
+// so the columns need each other only in its total (row by row, each non-zero exponent took a CTA-wide FP64 sum and
+// three barriers).
 __device__ void conj_weyl(Smem& s, const Ctx& C, const int8_t* xz, int* acc_x, int* acc_z, int* acc_r) {
   const int n = C.n, d = C.d;
   if (threadIdx.x == 0) s.ival[2] = 0;

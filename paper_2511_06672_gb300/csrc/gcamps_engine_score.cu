@@ -83,7 +83,7 @@ __device__ void gram_chunked(const Grp& g, const double2* theta, int cl, int cr,
 
 // Every class of one theta at once: CTA k < K takes the exact FP64 scores of class k, CTA K + k its FP32 screen and
 // estimate, into rows of kMaxK doubles (KnownScore).  The classes are independent, and 90 CTAs on 152 SMs take the
-// time of one: at m = 81 2 ms instead of 38 ms for the classes in turn on a cluster of 4.  theta', the Gram and the
+// time of one: 1.6 ms at m = 75 instead of 42 for the classes in turn on a cluster of 4.  theta', the Gram and the
 // reduction's scratch live in dynamic shared memory (kGridMax entries of theta).  Below kGridWarpM rows a CTA is one
 // warp (the steps of a reduction of so few rows fit one).
 constexpr int kGridMax = 81 * 81, kGridWarpM = 10, kGridWidth = 32;
@@ -194,7 +194,7 @@ cudaError_t launch_grid(const Engine& e, const double2* th, int cl, int cr, doub
   const size_t bytes = std::max(exact, est);
   const bool warp = m < kGridWarpM;
   auto kern = warp ? k_score_grid_warp : k_score_grid;
-  if (bytes > 16384) {   // with the static part it may exceed the 48 KB a kernel gets unasked
+  if (bytes + sizeof(Smem) > 48 * 1024) {   // more than a kernel gets unasked
     const cudaError_t a = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (a != cudaSuccess) return a;
   }
