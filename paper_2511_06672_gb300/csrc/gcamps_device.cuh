@@ -1696,8 +1696,9 @@ __device__ void move_center(Smem& s, const Ctx& C, int target) {
 // and base coefficients c_m in s.coef[0..d), applied to the circuit's MPS as an MPO of bond dimension
 // d that is diagonal in m, over the support span [f, l] of P, then [f, l] recompressed (Sec. 2.4).
 // (X^a Z^b)_{s s'} = omega^{b s'} delta_{s, s'+a}, so each MPO tensor is a gather with phases.
-// record: this is the circuit's non-Clifford step (span, string and counters are kept); the adjoint
-// passes false.  The identity string (f > l) sets EINVAL.
+// record: this is the circuit's non-Clifford step (span, string and counters are kept, and the state keeps norm 1
+// under truncation); the adjoint passes false: its O psi has a norm of its own, which the gradient is linear in (for
+// d = 3 O = (W + W^dag) / 2 has eigenvalues 1 and -1/2).  The identity string (f > l) sets EINVAL.
 // lead: the leader's shared memory when the other CTAs of the cluster serve cluster-Jacobi requests during
 // the step (run_op); null for a leader-only compression
 __device__ __noinline__ void mpo_apply(Smem& s, const Ctx& C, const uint8_t* row, int r, bool record,
@@ -1804,7 +1805,7 @@ __device__ __noinline__ void mpo_apply(Smem& s, const Ctx& C, const uint8_t* row
     for (int j = f; j < l; ++j) move_right(s, C, j);
     double disc = 0;
     for (int j = l; j > f; --j) {
-      disc += move_left(s, C, j, C.e->chi_max, true, lead);
+      disc += move_left(s, C, j, C.e->chi_max, record, lead);
       note_chi(C, C.dims[j]);
     }
     if (threadIdx.x == 0) {
