@@ -100,11 +100,19 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) k_adjoint(Engine e, int cf
     s.coef[d - 1].x += 0.5;   // P^(d-1) = P^dag
   }
   __syncthreads();
+  const int K = F.meta[M_NSNAP];
+  const int ndec = F.meta[M_NDEC];
+  // P^(d-1) is P^dag because W^d = 1, but for d = 2 a string with an odd number of X Z factors has W^2 = -1: it
+  // is anti-Hermitian, O = 0, and so is every derivative
+  int ny = 0;
+  for (int j = 0; j < n; ++j) ny += xz[j] * xz[n + j];
+  if (d == 2 && (ny & 1)) {
+    for (int i = threadIdx.x; i < K * d; i += blockDim.x) grad[i] = 0.0;
+    return;
+  }
   bool has_w = false;
   for (int j = 0; j < n; ++j) has_w |= (row[j] | row[n + j]) != 0;
   if (has_w) mpo_apply(s, B, row, ar, false);
-  const int K = F.meta[M_NSNAP];
-  const int ndec = F.meta[M_NDEC];
   for (int k = K - 1; k >= 0 && B.meta[M_STATUS] == 0; --k) {
     const int* hd = e.snap_hdr + ((long long)cf * e.snap_max + k) * kSnapHdr;
     const int dec0 = hd[3];

@@ -61,3 +61,17 @@ def test_gradient_of_evolved_strings(G, d, n, layers, ngates, seed, disentangle)
         assert np.max(np.abs(grad - rgrad)) < GRAD_TOL
     assert largest > 0.1
     sim.close()
+
+
+@pytest.mark.parametrize("n,layers,ngates,seed", [(6, 6, 8, 3), (11, 8, 9, 2)])
+def test_strings_with_an_odd_number_of_y_factors_have_gradient_zero(G, n, layers, ngates, seed):
+    """For d = 2 such a string (phase 1) is anti-Hermitian: Re <W>, the mean of (W + W^dag) / 2 = 0, is 0 for every
+    phase."""
+    gates, sim = _run(G, 2, n, layers, ngates, seed, True)
+    odd = [(x, z) for x, z in _evolved(gates, n, 2) if int(np.sum(x * z)) % 2]
+    assert odd
+    for x, z in odd:
+        val, grad = sim.expect_gradient(x, z)
+        assert abs(val) < VALUE_TOL
+        assert np.max(np.abs(grad)) < GRAD_TOL
+    sim.close()
