@@ -185,17 +185,29 @@ __global__ void __launch_bounds__(kThreads) k_score_choice(Engine e, const doubl
   }
 }
 
+// Dynamic shared memory of the scores of a theta with sides m <= M: the exact ones' (Gram, tridiagonal, a chunk of
+// theta'), the estimates' (theta, theta' and the Gram in FP32, three arrays of m).
+constexpr size_t grid_bytes(int m, int M) {
+  const size_t exact = (size_t)(m * m + m + m * ((M < kGridWidth ? M : kGridWidth) | 1)) * sizeof(double2);
+  const size_t est = (size_t)(2 * m * M + m * m + 3 * m) * sizeof(float2);
+  return exact > est ? exact : est;
+}
+// The most that any theta needs: m M <= kGridMax and m <= M, so no term is larger than at m = M = 81.
+constexpr int kGridSide = 81;
+constexpr size_t kGridBytes = grid_bytes(kGridSide, kGridSide);
+static_assert(kGridSide * kGridSide == kGridMax && kGridBytes + sizeof(Smem) <= 227 * 1024, "fits a CTA");
+
 // k_score_grid and k_score_choice for a theta of at most kGridMax entries; known: kKnownRows kMaxK doubles.
 cudaError_t launch_grid(const Engine& e, const double2* th, int cl, int cr, double* known, double* s2, double* vn,
                         int* choice, bool status, cudaStream_t st) {
   const int rows = cl * e.d, cols = e.d * cr, m = std::min(rows, cols), M = std::max(rows, cols);
-  const size_t exact = (size_t)(m * m + m + m * (std::min(M, kGridWidth) | 1)) * sizeof(double2);
-  const size_t est = (size_t)(2 * rows * cols + m * m + 3 * m) * sizeof(float2);
-  const size_t bytes = std::max(exact, est);
+  const size_t bytes = grid_bytes(m, M);
   const bool warp = m < kGridWarpM;
   auto kern = warp ? k_score_grid_warp : k_score_grid;
-  if (bytes + sizeof(Smem) > 48 * 1024) {   // more than a kernel gets unasked
-    const cudaError_t a = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  // more than a kernel gets unasked: the limit belongs to the kernel, not to the launch, so every call sets the same
+  // one (with its own size a call on another thread could lower it between this one's set and its launch)
+  if (bytes + sizeof(Smem) > 48 * 1024) {
+    const cudaError_t a = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGridBytes);
     if (a != cudaSuccess) return a;
   }
   kern<<<2 * e.K, warp ? 32 : kThreads, bytes, st>>>(e, th, cl, cr, known);
