@@ -340,8 +340,7 @@ int gcamps_get_profile(gcamps_t* h, int circuit, int64_t* out, int32_t cap, int3
  * FP64 where evaluated[k] = 1, else the FP32 screening value, within 4 eta sqrt(m) + 4 eta of the exact
  * one with eta < 3 (d^3 + 6 d + max side) 2^-24), vn[k] (von Neumann entropy, valid where
  * evaluated[k] = 1 except for classes scored by Renyi-2 alone under score_kind 1, which read NaN;
- * the bounds excluded the others; where the classes that make theta a product across the bond decided the
- * visit, those are the evaluated ones and their vn is their S2, within tie_tol / 2 of the entropy);
+ * the bounds excluded the others; class 0, the identity, is always evaluated);
  * K = gcamps_num_candidates(d) entries each; any pointer may be NULL. */
 int gcamps_get_last_scores(gcamps_t* h, int circuit, double* s2, double* vn, uint8_t* evaluated);
 /* Two-site tensor theta scored at the last bond visit (Sec. 3): shape[0..1] = (chi_l, chi_r); theta receives the

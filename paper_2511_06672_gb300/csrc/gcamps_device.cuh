@@ -246,8 +246,9 @@ struct Smem {
   double2 zdiag[kZCols];      // QR: diagonal of R
   double zbeta[kZCols];       // QR: reflector scalars
   int zperm[kZCols];
-  int npure, pure;            // select_class: classes of the purity test, and whether it decided (leader)
+  int npure, pure;            // select_class: classes of the purity test; whether it decided, 2 with exact scores (leader)
   int vbond;                  // bond of the visit the cluster serves next, -1 to leave the sweeps (leader)
+  int readable;               // whether its scores can be read after the call: a Readable (leader)
   uint8_t clean[kMaxN];       // bond b: the state around it is the one its last visit left (leader, disentangle)
   // the leader's counters of the launch (load_counters): one thread adds to them several times per visit, and the
   // others wait for it (in global memory the decision phase of a small visit took 4.9 kcycles, here 1.4)
@@ -3429,6 +3430,9 @@ __device__ __forceinline__ bool pure_choice(Smem& s, const Ctx& C, int m, int M)
   return true;
 }
 
+// A visit's scores stay readable (gcamps_get_last_scores) if it is the call's last one: known beforehand, or if it
+// applies nothing (the sweep's last bond when no bond before it took a class).
+enum Readable { kNotReadable = 0, kReadableIfIdle = 1, kReadable = 2 };
 // search: a disentangler visit; false for the scoring entry points, which report how many classes the
 // bounds alone leave.
 __device__ int select_class(Smem& s, Smem* lead, const Ctx& C, const double2* theta, int cl, int cr, int* nev_out,
@@ -3481,9 +3485,27 @@ __device__ int select_class(Smem& s, Smem* lead, const Ctx& C, const double2* th
       cluster_sync();
       if (leader && threadIdx.x < 32) {
         const bool done = pure_choice(s, C, m, rows < cols ? cols : rows);
-        if (threadIdx.x == 0) s.pure = done;
+        // scores that can be read afterwards hold the exact entropies of the identity and of every listed class
+        if (threadIdx.x == 0) {
+          s.pure = done;
+          if (done && (s.readable == kReadable || (s.readable == kReadableIfIdle && s.ival[4] == 0))) {
+            int cnt = s.npure;
+            if (s.list[0] != 0) {   // ascending
+              for (int t = cnt++; t > 0; --t) s.list[t] = s.list[t - 1];
+              s.list[0] = 0;
+            }
+            s.nlist = cnt;
+            s.ival[5] += cnt;
+            s.ival[7] += cnt;
+            s.pure = 2;
+          }
+        }
       }
       cluster_sync();
+      if (lead->pure == 2) {
+        score_classes(s, lead, C, theta, cl, cr, lead->list, lead->nlist, kExact);
+        cluster_sync();
+      }
       prof_lap(C, P_EXACT, tp);
       if (lead->pure) {
         if (!leader) return -1;
@@ -3724,9 +3746,9 @@ __device__ void serve_visits(Smem& s, Smem* lead, const Ctx& C) {
   }
 }
 
-// One bond visit, on the leader.  must_score: the visit's scores are readable afterwards, so they are taken even
-// where the decision is known.
-__device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, bool must_score, int* accepted) {
+// One bond visit, on the leader.  readable: where the visit's scores may be read afterwards, they are taken even if
+// the decision is known.
+__device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, Readable readable, int* accepted) {
   const Engine& e = *C.e;
   const int d = C.d, dd = d * d;
   double2* theta = C.scr + e.sl.theta;
@@ -3749,7 +3771,7 @@ __device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, b
   // its last visit but unitaries on one side of the pair's two sites, which leave every class's score as it was
   // (the classes of Q theta are those of theta, so after applying the best one the identity is the best).  The
   // QR move is what a scored visit would do: the rank of the first kind is 1, the clean mark holds the second's.
-  if (!replay && !must_score && chim <= cap && (chim == 1 || s.clean[i])) {
+  if (!replay && readable == kNotReadable && chim <= cap && (chim == 1 || s.clean[i])) {
     if (threadIdx.x == 0) {
       C.stats[S_BONDS] += 1;
       C.stats[S_CANDS] += C.K;
@@ -3776,7 +3798,8 @@ __device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, b
     s.dval[3] = vn_est_bound(d, m, rows < cols ? cols : rows);
     s.rank0 = -1;
     s.vbond = i;
-    s.ival[7] = 0;   // 1: the purity test decided
+    s.readable = readable;
+    s.ival[7] = 0;   // the purity test decided: 1 + the exact entropies taken all the same
   }
   // Splits with many Jacobi columns run their rotations on the whole cluster: the other CTAs wait for the
   // leader's choice (a QR move or such a split) at one more cluster barrier.
@@ -3817,7 +3840,7 @@ __device__ void visit_bond(Smem& s, Smem* lead, const Ctx& C, int i, bool ltr, b
     class_flops(d, rows, cols, gram, tri);
     // exact evaluations, FP64 (Renyi-2 scores and the purity test need no eigenvalues, but for the identity's
     // of the former)
-    C.dstats[1] += e.score_kind == 1 ? nev * gram + tri : nev * (s.ival[7] ? gram : gram + tri);
+    C.dstats[1] += e.score_kind == 1 ? nev * gram + tri : nev * gram + (s.ival[7] ? s.ival[7] - 1 : nev) * tri;
     if (m > kPruneMin) C.dstats[4] += C.K * (gram + tri);   // every class scored exactly (the algorithm)
     if (m > kPruneMin) C.dstats[2] += C.K * gram;                // FP32 screen of every class
     record_decision(C, i, s.ival[4]);
@@ -3954,9 +3977,9 @@ __device__ void disentangle(Smem& s, Smem* lead, const Ctx& C, int sweep_cap, in
           break;
         }
         const int i = ltr ? f + t : l - 1 - t;
-        const bool last = (t == l - f - 1 && (acc == 0 || sweep + 1 == max_sweeps)) ||
-                          (visit_cap > 0 && visits + 1 >= visit_cap);
-        visit_bond(s, lead, C, i, ltr, last, &acc);
+        const bool end = t == l - f - 1;   // of the sweep
+        const bool last = (end && sweep + 1 == max_sweeps) || (visit_cap > 0 && visits + 1 >= visit_cap);
+        visit_bond(s, lead, C, i, ltr, last ? kReadable : (end && acc == 0 ? kReadableIfIdle : kNotReadable), &acc);
         ++visits;
       }
       if (capped) break;
