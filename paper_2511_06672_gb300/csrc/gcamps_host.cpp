@@ -1127,14 +1127,24 @@ int gcamps_batch_get_bond_dims(gcamps_t* h, int circuit, int32_t* chi) {
   if (rc) return rc;
   if (!chi) return fail(h, GCAMPS_EINVAL, "null output");
   const int n = h->nq[circuit];
-  // the circuit's bond dimensions up to the status words, which follow those of the last circuit: one copy, one wait
   const int* first = h->e.dims + (long long)circuit * (h->e.n + 1);
-  const size_t upto = (const char*)(h->e.meta + (size_t)h->e.batch * gcx::M_COUNT) - (const char*)first;
-  std::vector<int> dims(upto / sizeof(int));
-  GC_CUDA(h, cudaMemcpyAsync(dims.data(), first, upto, cudaMemcpyDeviceToHost, h->stream));
+  const int* status = h->e.meta;                                      // behind the last circuit's dimensions
+  const size_t status_words = (size_t)h->e.batch * gcx::M_COUNT;
+  // One copy up to the end of the status words, unless more than 512 KB of other circuits' dimensions lie between (at
+  // 4096 circuits of 64 qudits, 1 MB before the first: 47.6 us in one copy, 33.2 in two; half of that: 35.7 and 33.7;
+  // a quarter: 23.0 and 25.2).
+  const bool one = (const char*)status - (const char*)first <= (1 << 19);
+  const size_t row = one ? status - first : (size_t)n + 1;
+  std::vector<int> words(row + status_words);
+  if (one) {
+    GC_CUDA(h, cudaMemcpyAsync(words.data(), first, words.size() * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  } else {
+    GC_CUDA(h, cudaMemcpyAsync(words.data(), first, row * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    GC_CUDA(h, cudaMemcpyAsync(words.data() + row, status, status_words * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  }
   GC_CUDA(h, cudaStreamSynchronize(h->stream));
-  for (int j = 0; j < n - 1; ++j) chi[j] = dims[j + 1];
-  return check_status(h, dims.data() + (h->e.meta - first));
+  for (int j = 0; j < n - 1; ++j) chi[j] = words[j + 1];
+  return check_status(h, words.data() + row);
 }
 
 // The single-circuit forms of the contract (circuit 0 of the handle).
