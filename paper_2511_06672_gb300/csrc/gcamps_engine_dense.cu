@@ -177,7 +177,8 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
   return z ^ (z >> 31);
 }
 
-// psi(y) for the requested labels (all if ys is null), on one cluster.  work: 4 dim entries, then one per CTA.  The
+// psi(y) for the requested labels (all if ys is null), on one cluster, and behind them 1 if the state's bonds exceed their
+// Schmidt bounds (nothing else is written then), else 0.  work: 4 dim entries, then one per CTA.  The
 // phase of C is the one that gives C|0> = P v / |P v|, P the projector on the stabilizer rows' +1 eigenvector and v a
 // fixed hashed vector: that of <C 0|v>, so |0> goes through the same passes.
 template <int D>
@@ -197,8 +198,9 @@ __device__ void dense_body(DenseWord& w, Smem& s, const Engine& e, int c, int di
   int rows = 1, chi = 1;
   bool fits = true;   // the same on every CTA
   for (int j = 0, r = D; j < n; ++j, r *= D) fits = fits && (long long)r * C.dims[j + 1] <= dim;
-  if (!fits) {        // not a state this engine leaves: no readout of it
-    for (int t = gt; t < nys; t += gn) out[t] = cz();
+  // a state beyond them is none that this engine leaves: not read, and the caller is told by the entry behind the outputs
+  if (gt == 0) out[nys] = make_double2(fits ? 0.0 : 1.0, 0.0);
+  if (!fits) {
     cluster_sync();
     return;
   }

@@ -1038,7 +1038,8 @@ static int statevector_impl(gcamps_t* h, int circuit, const int32_t* ys, long lo
     dim *= d;
     if (dim > (1LL << 20)) return fail(h, GCAMPS_EINVAL, "d^n above 2^20: dense readout not supported");
   }
-  // the workspace (64 MB at 2^20 entries), the outputs and the label stay with the handle
+  // the workspace (64 MB at 2^20 entries), the outputs (16 MB), the entry behind them and the label stay with the handle;
+  // the label (nys = 1) lies beyond the entry behind its one output
   const size_t work_bytes = (gcx::statevector_work(dim) + 255) / 256 * 256;
   const size_t bytes = work_bytes + (size_t)dim * sizeof(double2) + 256;
   if (bytes > h->dense_cap) {
@@ -1057,11 +1058,15 @@ static int statevector_impl(gcamps_t* h, int circuit, const int32_t* ys, long lo
   cudaError_t ce = cudaSuccess;
   if (ys) ce = cudaMemcpyAsync(ys_dev, ys, (size_t)nys * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream);
   if (ce == cudaSuccess) ce = gcx::launch_statevector(h->e, circuit, out, dim, ys_dev, nys, base, h->stream);
-  std::vector<double2> host((size_t)nys);
+  std::vector<double2> host((size_t)nys + 1);   // the entry behind the outputs: whether the state could be read
   if (ce == cudaSuccess)
-    ce = cudaMemcpyAsync(host.data(), out, (size_t)nys * sizeof(double2), cudaMemcpyDeviceToHost, h->stream);
+    ce = cudaMemcpyAsync(host.data(), out, host.size() * sizeof(double2), cudaMemcpyDeviceToHost, h->stream);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(h->stream);
   if (ce != cudaSuccess) return cuda_fail(h, ce, "statevector");
+  if (host[(size_t)nys].x != 0.0) {
+    const int rc = device_status(h);
+    return rc ? rc : fail(h, GCAMPS_EINVAL, "bond dimensions above the Schmidt bounds: no dense readout");
+  }
   for (long long i = 0; i < nys; ++i) {
     re[i] = host[(size_t)i].x;
     im[i] = host[(size_t)i].y;

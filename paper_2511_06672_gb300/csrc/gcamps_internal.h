@@ -132,7 +132,7 @@ cudaError_t launch_single(const Engine& e, const gcamps_op& op, cudaStream_t st)
 cudaError_t launch_reset(const Engine& e, cudaStream_t st);
 cudaError_t launch_expect(const Engine& e, int circuit, const int8_t* xz_dev, double2* out_dev,
                           cudaStream_t st);
-// Dense readout (gcamps_engine_dense.cu): work holds statevector_work(d^n) bytes.
+// Dense readout (gcamps_engine_dense.cu): work holds statevector_work(d^n) bytes, out_dev nys + 1 entries.
 size_t statevector_work(long long dim);
 cudaError_t launch_statevector(const Engine& e, int circuit, double2* out_dev, long long dim,
                                const int32_t* ys_dev, long long nys, void* work, cudaStream_t st);
