@@ -58,7 +58,7 @@ def arith_peaks():
     except (OSError, ValueError, KeyError):
         return FP64_NOMINAL_TFLOPS, FP32_NOMINAL_TFLOPS, "nominal (no measurement committed)"
 ENGINE_SRCS = [os.path.join(ROOT, "paper_2511_06672_gb300", "csrc", f)
-               for f in ("gcamps_device.cuh", "gcamps_engine.cu", "gcamps_internal.h")]
+               for f in ("gcamps_device.cuh", "gcamps_engine.cu", "gcamps_internal.h", "gcamps_roots.cuh")]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_run_dram_bench_workload.txt")
 
 

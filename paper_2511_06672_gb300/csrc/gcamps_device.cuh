@@ -34,6 +34,7 @@
 #include <cstdint>
 
 #include "gcamps_internal.h"
+#include "gcamps_roots.cuh"
 
 namespace gcx {
 namespace {
@@ -166,23 +167,6 @@ __device__ __forceinline__ void group_sum2(double& a, double& b, int G) {
 }
 // Lanes that share a column of m entries: one pass over it where it fits a warp.
 __device__ __forceinline__ int lanes_for(int m) { return m <= 8 ? 8 : (m <= 16 ? 16 : 32); }
-
-// 1 / sqrt(a) for a in the normal range: the hardware's approximation y and one step of the cubically convergent
-// iteration y (1 + e/2 + 3 e^2/8), e = 1 - a y^2: five FP64 instructions of 64 cycles.  The first step's error
-// 5 e^3 / 16 is below 2^-56 for an approximation good to 2^-18.
-__device__ __forceinline__ double rsqrt_fast(double a) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-  const double e = fma(-(a * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-// 1 / a for a in the normal range, by y (1 + e + e^2), e = 1 - a y.
-__device__ __forceinline__ double rcp_fast(double a) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-  const double e = fma(-a, y, 1.0);
-  return fma(y * e, 1.0 + e, y);
-}
 
 // -------------------------------------------------------------------------- per-CTA workspace
 // One Clifford on (q0, q1) (q1 = q0 for one qudit): the exponents of its generator images, generator k's at
