@@ -357,8 +357,8 @@ int gcamps_get_decisions(gcamps_t* h, int circuit, int32_t* pairs, int32_t cap, 
  * s2[k] = Renyi-2 entropy and vn[k] = von Neumann entropy (natural log) of the Schmidt spectrum of
  * Q_k theta across (a, s) | (t, b), K = gcamps_num_candidates(d) entries each.  Runs the same device
  * code as gcamps_disentangle (every class evaluated here).  choice (may be NULL) receives the
- * class the disentangler would apply to this theta (0 = none) and how many exact entropies its
- * Renyi-2 pruning evaluated.  Synchronising. */
+ * class the disentangler would apply to this theta (0 = none) and how many exact entropies its bounds
+ * leave to evaluate (a count of the pruning; all K are evaluated in this call).  Synchronising. */
 int gcamps_score_theta(gcamps_t* h, int chi_l, int chi_r, const double* theta, double* s2, double* vn,
                        int32_t* choice);
 
@@ -390,7 +390,7 @@ int gcamps_estimate_theta(gcamps_t* h, int chi_l, int chi_r, const double* theta
  * as in gcamps_score_theta.  choice_dev: 3 int32, the class the von Neumann disentangler (score_kind 0,
  * rank threshold of cutoff 0) would apply (0 = none; a class is applied only if it lowers the entropy by
  * more than tie_tol, ties to the lowest index; handles made with score_kind 1 or 2 can choose otherwise),
- * the number of exact entropies its Renyi-2 pruning evaluated, and the device status of the call
+ * the number of exact entropies its bounds leave to evaluate (all K are evaluated here), and the device status of the call
  * (0 or a GCAMPS_E* code; the eigenvalue search runs a fixed number of steps, so 0 in practice).  cuda_stream: the cudaStream_t
  * to run on, NULL for the default stream.  Asynchronous: the outputs are valid once the stream has
  * passed this call.
@@ -398,8 +398,7 @@ int gcamps_estimate_theta(gcamps_t* h, int chi_l, int chi_r, const double* theta
  * The first call on a device, with that device current, does a one-time set-up: it looks up the
  * device address of the static array and copies the class tables into static device memory
  * (synchronous copies).  Make that first call before any stream capture.  All calls on a device
- * share the one array and it keeps the last call's contents; each call clears the words that must
- * start at zero itself.  Calls whose kernels overlap on the GPU (several streams, or several host
+ * share the one array and it keeps the last call's contents, which no later call reads.  Calls whose kernels overlap on the GPU (several streams, or several host
  * threads at once) race on the array and give wrong results: serialise them.
  * Returns GCAMPS_OK; GCAMPS_EINVAL (d not 2 or 3, a null pointer, chi < 1, tie_tol < 0 or NaN);
  * GCAMPS_ESIZE; GCAMPS_ECUDA (set-up or launch failed). */

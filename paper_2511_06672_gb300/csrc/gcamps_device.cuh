@@ -190,8 +190,10 @@ struct Smem {
   double vbd[kMaxK];          // its error bound: |vest - S_vN| <= vbd (cluster leader)
   uint8_t estd[kMaxK];        // vest[k] valid
   int rk[kMaxK];              // weight rank of each exactly evaluated class (cluster leader)
-  // Scoring and the small factorisations never overlap on a CTA (a cluster barrier lies between): they share the
-  // space, which leaves the SM's L1 to the scratch in global memory.
+  // Scoring, the small factorisations and the gate tables never overlap on a CTA: they share the space, which leaves the
+  // SM's L1 to the scratch in global memory.  Only the CTA's own threads use it.  Its scoring ends at the cluster
+  // barrier after it; a factorisation and a table each end at their last CTA barrier (a fold's table comes right before
+  // its visit's split, a gate list's tables right after a centre move), and the next use starts behind that.
   union {
     struct {
       double wtri[kWarps][64];    // per warp: tridiagonal diagonal [0, 32) | off-diagonal squared [32, 64)
